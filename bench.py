@@ -56,7 +56,7 @@ def measured_peak_gbs():
     return 6800.0, "fallback"
 
 
-KERNEL_SOURCES = ("lbm_common.cuh", "lbm_kernels.cuh", "lbm_kernels_async.cuh", "lbm_kernels_chunk.cuh",
+KERNEL_SOURCES = ("lbm_common.cuh", "lbm_exptab.cuh", "lbm_math.cuh", "lbm_kernels.cuh", "lbm_kernels_async.cuh", "lbm_kernels_chunk.cuh",
                   "lbm_kernels_moment.cuh", "lbm_kernels_tma.cuh", "lbm_lattice_inst.cuh")
 
 

@@ -9,6 +9,8 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include "lbm_exptab.cuh"
+
 namespace lbm {
 
 constexpr int Q = 19;
@@ -71,8 +73,11 @@ __device__ __forceinline__ T psi_of(T n, const EosParams& e);
 
 template <>
 __device__ __forceinline__ double psi_of<double>(double n, const EosParams& e) {
-  if (e.kind == kPsiOneMinusExp) return -expm1(-n);
-  if (e.kind == kPsiExpInv) return exp(-1.0 / n);
+  if (e.kind == kPsiOneMinusExp) return exp_arg_ok(n) ? exp_neg_table<true>(n) : -expm1(-n);
+  if (e.kind == kPsiExpInv) {
+    const double y = 1.0 / n;
+    return exp_arg_ok(y) ? exp_neg_table<false>(y) : exp(-y);
+  }
   // Carnahan-Starling mapped: psi = sqrt(2 (p_CS - n c_s^2) / (G c_s^2))
   const double q = e.b * n * 0.25;
   const double om = 1.0 - q;

@@ -22,27 +22,9 @@
 #pragma once
 
 #include "lbm_common.cuh"
+#include "lbm_math.cuh"
 
 namespace lbm {
-
-// shell weights W(|xi|^2) of the forcing stencils (Sec. II; wider stencils
-// are the isotropic ones the paper cites): 0 where a vector is not used
-template <int ST>
-__host__ __device__ constexpr double shell_weight(int s) {
-  if (ST == 4) return s == 1 ? 1.0 / 6.0 : (s == 2 ? 1.0 / 12.0 : 0.0);
-  if (ST == 6)
-    return s == 1 ? 2.0 / 15.0 : s == 2 ? 1.0 / 15.0 : s == 3 ? 1.0 / 60.0 : s == 4 ? 1.0 / 120.0 : 0.0;
-  // E8
-  return s == 1 ? 4.0 / 45.0
-       : s == 2 ? 1.0 / 21.0
-       : s == 3 ? 2.0 / 105.0
-       : s == 4 ? 5.0 / 504.0
-       : s == 5 ? 1.0 / 315.0
-       : s == 6 ? 1.0 / 630.0
-       : s == 8 ? 1.0 / 5040.0
-       : 0.0;
-}
-template <int ST> constexpr int stencil_radius() { return ST == 4 ? 1 : 2; }
 
 // per-CTA reduction record of the field-observable pass
 struct FieldPartial {
@@ -77,32 +59,6 @@ struct StepShape {
   static constexpr size_t pops_bytes = sizeof(T) * NP * Q * NT;
   static constexpr size_t smem_bytes = ring_bytes + pops_bytes;
 };
-
-// Mirror-exact summation.  The box, the droplet and its initial profile are
-// symmetric under the three reflections x -> -x, y -> -y, z -> -z about the centre
-// node, and so is the exact dynamics; floating-point sums keep that symmetry only
-// if each reflection maps every sum onto the same operations.  A reflection
-// permutes the populations (x: 1<->2, 7<->10, 8<->9, 11<->14, 12<->13; y: 3<->4,
-// 7<->9, 8<->10, 15<->18, 16<->17; z: 5<->6, 11<->13, 12<->14, 15<->17, 16<->18), so
-// the sums below add opposite pairs first and then exactly the pair sums a
-// reflection swaps; a + b = b + a and a - b = -(b - a) hold exactly, so a mirrored
-// state gives bitwise mirrored densities, momenta and forces, the drop's centre of
-// mass stays on the centre node, and rounding (FP16 storage above all) cannot push
-// the drop off it.
-//
-// sum of the nine opposite-pair sums g_i + g_ibar, grouped by the reflections
-template <typename T>
-__device__ __forceinline__ T pair_sum9(T p12, T p34, T p56, T p78, T p910, T p1112, T p1314, T p1516, T p1718) {
-  return ((p12 + p34) + p56) + (((p78 + p910) + (p1112 + p1314)) + (p1516 + p1718));
-}
-
-// density: rest population plus the mirror-exact sum of the pair sums (the order
-// is fixed, so every kernel forms bitwise the same density)
-template <typename T>
-__device__ __forceinline__ T sum19(const T* v) {
-  return v[0] + pair_sum9<T>(v[1] + v[2], v[3] + v[4], v[5] + v[6], v[7] + v[8], v[9] + v[10],
-                             v[11] + v[12], v[13] + v[14], v[15] + v[16], v[17] + v[18]);
-}
 
 // Pull the 19 populations of every node of one padded plane (tile + R halo),
 // form psi into the ring slot, park the interior populations if asked.
@@ -143,82 +99,21 @@ __device__ __forceinline__ void load_plane(const LatticeDesc& d, int x0, int y0,
   }
 }
 
-// Shan-Chen force (Eq. (8)) from psi planes in shared memory.  planes[dz + R]
+// Shan-Chen force (sc_force_at) from psi planes in shared memory.  planes[dz + R]
 // points at the node's own position in the psi plane at offset dz; rows are PX
-// apart.  The stencil is summed through the differences D(xi) = psi(x + xi) -
-// psi(x - xi), so that two psi values cancel before they are scaled: a uniform
-// region gives exactly F = 0 and the rounding error scales with F, not with the
-// psi values.  (Summing the 18 terms one by one in raster order lets FP32 rounding
-// build a spurious force that grows the density error of a 1000-step droplet run
-// tenfold.)
-// Mirror-exact order: component a of the force is, per shell, a sum over the
-// orbits of the stencil vectors with xi_a > 0 under the two reflections that
-// leave axis a alone -- {(xi_a, +-b, +-c)} -- each orbit summed as
-// ((D(a,b,c) + D(a,-b,c)) + (D(a,b,-c) + D(a,-b,-c))); the shells are then
-// weighted and added in a fixed order.  A reflection of the field maps every
-// orbit sum onto itself (reordered by exactly commuting additions) or onto its
-// negative, so mirrored psi gives a bitwise mirrored force (see sum19).
+// apart.
 // OWN: own[dz + R] holds psi of the node's own column at offset dz (the caller
 // formed those values and kept them in registers); differences along the node's
 // own column take them from there instead of from shared memory.
-template <typename T, int ST, int PX, bool OWN>
-__device__ __forceinline__ T sc_diff(const T* const* planes, const T* own, int dx, int dy, int dz) {
-  constexpr int R = stencil_radius<ST>();
-  if (OWN && dx == 0 && dy == 0) return own[R + dz] - own[R - dz];
-  return planes[R + dz][dy * PX + dx] - planes[R - dz][-dy * PX - dx];
-}
-
-template <typename T, int ST, int PX, bool OWN>
-__device__ __forceinline__ T sc_force_axis(const T* const* planes, const T* own, int axis) {
-  constexpr int R = stencil_radius<ST>();
-  T F = (T)0;
-  bool any_shell = false;
-#pragma unroll
-  for (int sh = 1; sh <= 3 * R * R; ++sh) {
-    const double W = shell_weight<ST>(sh);
-    if (W == 0.0) continue;
-    T S = (T)0;
-    bool any = false;
-#pragma unroll
-    for (int a = 1; a <= R; ++a) {
-#pragma unroll
-      for (int b = 0; b <= R; ++b) {
-#pragma unroll
-        for (int c = 0; c <= R; ++c) {
-          if (a * a + b * b + c * c != sh) continue;
-          // the vector (a, b, c) in the frame of `axis`: a along it, b and c along the
-          // other two axes in increasing order
-          auto D = [&](int bb, int cc) {
-            return axis == 0 ? sc_diff<T, ST, PX, OWN>(planes, own, a, bb, cc)
-                 : axis == 1 ? sc_diff<T, ST, PX, OWN>(planes, own, bb, a, cc)
-                             : sc_diff<T, ST, PX, OWN>(planes, own, bb, cc, a);
-          };
-          T O;
-          if (b > 0 && c > 0) O = (D(b, c) + D(-b, c)) + (D(b, -c) + D(-b, -c));
-          else if (b > 0) O = D(b, 0) + D(-b, 0);
-          else if (c > 0) O = D(0, c) + D(0, -c);
-          else O = D(0, 0);
-          if (a != 1) O = (T)a * O;
-          S = any ? S + O : O;
-          any = true;
-        }
-      }
-    }
-    if (!any) continue;
-    F = any_shell ? F + (T)W * S : (T)W * S;
-    any_shell = true;
-  }
-  return F;
-}
-
 template <typename T, int ST, int PX, bool OWN = false>
 __device__ __forceinline__ void sc_force_pairs(const T* const* planes, T G, T& Fx, T& Fy, T& Fz,
                                                const T* own = nullptr) {
   constexpr int R = stencil_radius<ST>();
-  const T k = -G * (T)(1.0 / 3.0) * (OWN ? own[R] : planes[R][0]);
-  Fx = k * sc_force_axis<T, ST, PX, OWN>(planes, own, 0);
-  Fy = k * sc_force_axis<T, ST, PX, OWN>(planes, own, 1);
-  Fz = k * sc_force_axis<T, ST, PX, OWN>(planes, own, 2);
+  auto at = [&](int dx, int dy, int dz) {
+    if (OWN && dx == 0 && dy == 0) return own[R + dz];
+    return planes[R + dz][dy * PX + dx];
+  };
+  sc_force_at<T, ST>(at, at(0, 0, 0), G, Fx, Fy, Fz);
 }
 
 // Force at interior node (tx, ty) of the current plane from the psi ring;
@@ -235,97 +130,6 @@ __device__ __forceinline__ void sc_force(const typename Storage<P>::T* ring, con
 #pragma unroll
   for (int k = 0; k <= 2 * R; ++k) planes[k] = ring + slots[k] * (PX * PY) + (ty + R) * PX + (tx + R);
   sc_force_pairs<T, ST, PX>(planes, G, Fx, Fy, Fz);
-}
-
-// BGK + Guo collision of one node in shifted form, g_i = f_i - w_i n0:
-//   g*_i = (1 - omega) g_i + omega g_i^eq + F_i
-//   g_i^eq = w_i [dn + n (3 e.u + 9/2 (e.u)^2 - 3/2 u.u)]          Eq. (6)
-//   F_i    = (1 - omega/2) w_i [3 e.F + 9 (e.u)(e.F) - 3 u.F]       Eq. (5)
-// Opposite velocities share the even part; the odd part flips sign.
-// CLOSE_MASS: the collision conserves mass exactly (sum g*_i = dn), but the
-// rounded weights do not sum to exactly 1 (FP32: 1 + 1.5e-8), which would
-// add a systematic error proportional to n - n0 to every node every step; the
-// rest population is set to dn - sum_{i>0} g*_i instead (the same value in
-// exact arithmetic), so mass changes only by uncorrelated rounding.
-// UNIT_TAU: tau = 1 (the relaxation time the method uses); then 1 - omega = 0
-// and the post-collision populations depend on the old ones only through n, j.
-// SCALED: the outputs come multiplied by wscale, a power of two (FP16 storage's
-// 2^k), folded into the weights and the mass closure; a power-of-two factor
-// commutes with every rounding, so the values are bitwise those of the
-// unscaled collision times wscale.
-template <typename T, bool CLOSE_MASS, bool UNIT_TAU = false, bool SCALED = false>
-__device__ __forceinline__ void collide(T* g, T dn, T n, T ux, T uy, T uz, T Fx, T Fy, T Fz,
-                                        T omega_in, T wscale = (T)1) {
-  const T omega = UNIT_TAU ? (T)1 : omega_in;
-  const T uu = ux * ux + uy * uy + uz * uz;
-  const T uF = ux * Fx + uy * Fy + uz * Fz;
-  const T cg = (T)1 - (T)0.5 * omega;     // 1 - 1/(2 tau)
-  const T om1 = (T)1 - omega;
-  const T base = omega * (dn - (T)1.5 * n * uu) - (T)3 * cg * uF;
-  g[0] = UNIT_TAU ? (T)(1.0 / 3.0) * base : om1 * g[0] + (T)(1.0 / 3.0) * base;
-#pragma unroll
-  for (int i = 1; i < Q; i += 2) {
-    const T eu = (T)cx(i) * ux + (T)cy(i) * uy + (T)cz(i) * uz;
-    const T eF = (T)cx(i) * Fx + (T)cy(i) * Fy + (T)cz(i) * Fz;
-    const T wi = SCALED ? (T)wq(i) * wscale : (T)wq(i);
-    const T even = base + omega * (T)4.5 * n * eu * eu + (T)9 * cg * eu * eF;
-    const T odd = (T)3 * (omega * n * eu + cg * eF);
-    if (UNIT_TAU) {
-      g[i] = wi * (even + odd);
-      g[i + 1] = wi * (even - odd);
-    } else {
-      g[i] = om1 * g[i] + wi * (even + odd);
-      g[i + 1] = om1 * g[i + 1] + wi * (even - odd);
-    }
-  }
-  if (CLOSE_MASS) {
-    // pair sums first (their odd parts cancel), then the mirror-exact grouping
-    g[0] = (SCALED ? dn * wscale : dn) -
-           pair_sum9<T>(g[1] + g[2], g[3] + g[4], g[5] + g[6], g[7] + g[8], g[9] + g[10], g[11] + g[12],
-                        g[13] + g[14], g[15] + g[16], g[17] + g[18]);
-  }
-}
-
-// The unit-tau collision of `collide<T, true, true>` with each post-collision
-// population stored as soon as it is formed (store(i, g_i)): only the nine pair
-// sums stay live for the mass closure, not all nineteen values.  Same operations
-// in the same order, so the stored values are bitwise those of collide().
-template <typename T, typename Store>
-__device__ __forceinline__ void collide_unit_tau_store(T dn, T n, T ux, T uy, T uz, T Fx, T Fy, T Fz,
-                                                       Store store) {
-  const T uu = ux * ux + uy * uy + uz * uz;
-  const T uF = ux * Fx + uy * Fy + uz * Fz;
-  const T cg = (T)1 - (T)0.5 * (T)1;
-  const T base = (T)1 * (dn - (T)1.5 * n * uu) - (T)3 * cg * uF;
-  T p[9];
-#pragma unroll
-  for (int i = 1; i < Q; i += 2) {
-    const T eu = (T)cx(i) * ux + (T)cy(i) * uy + (T)cz(i) * uz;
-    const T eF = (T)cx(i) * Fx + (T)cy(i) * Fy + (T)cz(i) * Fz;
-    const T wi = (T)wq(i);
-    const T even = base + (T)1 * (T)4.5 * n * eu * eu + (T)9 * cg * eu * eF;
-    const T odd = (T)3 * ((T)1 * n * eu + cg * eF);
-    const T ga = wi * (even + odd), gb = wi * (even - odd);
-    store(i, ga);
-    store(i + 1, gb);
-    p[i / 2] = ga + gb;
-  }
-  store(0, dn - pair_sum9<T>(p[0], p[1], p[2], p[3], p[4], p[5], p[6], p[7], p[8]));
-}
-
-// density and momentum of one node: momentum from the differences of the nine
-// opposite pairs (1,2), (3,4), ..., (17,18) of the population order
-template <typename T>
-__device__ __forceinline__ void moments(const T* g, T& dn, T& jx, T& jy, T& jz) {
-  dn = sum19(g);
-  const T d12 = g[1] - g[2], d34 = g[3] - g[4], d56 = g[5] - g[6];
-  const T d78 = g[7] - g[8], d910 = g[9] - g[10], d1112 = g[11] - g[12];
-  const T d1314 = g[13] - g[14], d1516 = g[15] - g[16], d1718 = g[17] - g[18];
-  // x: 1 (+), 7 (+), 9 (+), 11 (+), 13 (+); y: 3, 7, 10, 15, 17 (+); z: 5, 11, 14, 15, 18 (+);
-  // the differences a reflection swaps are added (or subtracted) first: mirror-exact
-  jx = (d12 + (d78 + d910)) + (d1112 + d1314);
-  jy = (d34 + (d78 - d910)) + (d1516 + d1718);
-  jz = (d56 + (d1112 - d1314)) + (d1516 - d1718);
 }
 
 template <typename T>
@@ -406,11 +210,7 @@ lattice_kernel(LatticeDesc d, int zchunk, ObsArgs oa) {
         T dn, jx, jy, jz;
         moments(g, dn, jx, jy, jz);
         const T n = n0 + dn;
-        const T inv_n = (T)1 / n;
-        const T ux = (jx + (T)0.5 * Fx) * inv_n;
-        const T uy = (jy + (T)0.5 * Fy) * inv_n;
-        const T uz = (jz + (T)0.5 * Fz) * inv_n;
-        collide<T, true>(g, dn, n, ux, uy, uz, Fx, Fy, Fz, omega);
+        collide<T>(g, dn, n, jx, jy, jz, Fx, Fy, Fz, omega);
         S* __restrict__ dst = static_cast<S*>(d.dst);
 #pragma unroll
         for (int i = 0; i < Q; ++i) Storage<P>::store(dst + (long long)i * plane + node, g[i], scale);

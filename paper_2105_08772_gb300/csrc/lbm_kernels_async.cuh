@@ -181,11 +181,7 @@ __device__ __forceinline__ void async_process_item(const LatticeDesc& d, int zch
         T dn, jx, jy, jz;
         moments(g, dn, jx, jy, jz);
         const T n = n0 + dn;
-        const T inv_n = (T)1 / n;
-        const T ux = (jx + (T)0.5 * Fx) * inv_n;
-        const T uy = (jy + (T)0.5 * Fy) * inv_n;
-        const T uz = (jz + (T)0.5 * Fz) * inv_n;
-        collide<T, true, UNIT_TAU>(g, dn, n, ux, uy, uz, Fx, Fy, Fz, omega);
+        collide<T, UNIT_TAU>(g, dn, n, jx, jy, jz, Fx, Fy, Fz, omega);
         const int node = ((z0 + k) * ny + (y0 + ty)) * nx + (x0 + tx);
 #pragma unroll
         for (int i = 0; i < Q; ++i) dstp[i][node] = (S)g[i];

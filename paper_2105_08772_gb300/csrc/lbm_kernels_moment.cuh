@@ -284,21 +284,16 @@ __device__ __forceinline__ void moment_process_item(const LatticeDesc& d, int zc
       sc_force_pairs<T, ST, PX, true>(planes, G, Fx, Fy, Fz, pz);
       const T dn = mdn[R];       // plane qc = qd - 1 - R: R planes before the newest
       const T n = n0 + dn;
-      const T inv_n = (T)1 / n;
-      const T ux = (mjx[R] + (T)0.5 * Fx) * inv_n;
-      const T uy = (mjy[R] + (T)0.5 * Fy) * inv_n;
-      const T uz = (mjz[R] + (T)0.5 * Fz) * inv_n;
-      T g[Q];     // written, never read, by the unit-tau collision
-      // FP16: the collision returns the populations times the storage scale
-      collide<T, true, true, P == kF16>(g, dn, n, ux, uy, uz, Fx, Fy, Fz, (T)1, scale);
       const long long node = ((long long)(z0 + k) * ny + (y0 + ty)) * nx + (x0 + tx);
-      S* q = dst + node;   // population i's plane is i * plane further on
-#pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        if constexpr (P == kF16) *q = __float2half_rn(g[i]);   // already scaled
-        else Storage<P>::store(q, g[i], scale);
-        q += plane;
-      }
+      S* out = dst + node;
+      // each population is stored as soon as it is formed (FP16: the collision
+      // returns them times the storage scale)
+      collide_nodes<T, true, P == kF16>(dn, n, mjx[R], mjy[R], mjz[R], Fx, Fy, Fz, (T)1, scale,
+                                        [](int) { return (T)0; },
+                                        [&](int i, T v) {
+                                          if constexpr (P == kF16) out[i * plane] = __float2half_rn(v);
+                                          else out[i * plane] = v;
+                                        });
     }
 #pragma unroll
     for (int r = R; r > 0; --r) {

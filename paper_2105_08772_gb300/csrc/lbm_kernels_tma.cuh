@@ -483,13 +483,9 @@ __device__ __forceinline__ bool tma_process_item(const LatticeDesc& d, const Tma
       sc_force_pairs<T, ST, PX, true>(planes, G, Fx, Fy, Fz, pz);
       const T dn = mdn[R];
       const T n = n0 + dn;
-      const T inv_n = (T)1 / n;
-      const T ux = (mjx[R] + (T)0.5 * Fx) * inv_n;
-      const T uy = (mjy[R] + (T)0.5 * Fy) * inv_n;
-      const T uz = (mjz[R] + (T)0.5 * Fz) * inv_n;
       float* out = dst + (((long long)(z0 + k) * ny + (y0 + ty)) * nx + (x0 + tx));
-      collide_unit_tau_store<T>(dn, n, ux, uy, uz, Fx, Fy, Fz,
-                                [&](int i, T v) { out[i * plane] = v; });
+      collide_nodes<T, true, false>(dn, n, mjx[R], mjy[R], mjz[R], Fx, Fy, Fz, (T)1, (T)1,
+                                    [](int) { return (T)0; }, [&](int i, T v) { out[i * plane] = v; });
     }
 #pragma unroll
     for (int r = R; r > 0; --r) {
