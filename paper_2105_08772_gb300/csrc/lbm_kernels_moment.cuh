@@ -1,4 +1,6 @@
-// Unit-relaxation-time variant of the pipelined Shan-Chen step (FP32 / FP64).
+// Unit-relaxation-time variant of the pipelined Shan-Chen step (FP32 / FP64).  FP32 and
+// FP16 E4 boxes of 190000 nodes and more take the row kernel (lbm_kernels_row.cuh)
+// unless a z chunk is fixed; this one runs the rest.
 //
 // With tau = 1 the BGK update of Eq. (4) loses its f_i term:
 //     f*_i = f_i - (f_i - f_i^eq) + F_i = f_i^eq(n, u) + F_i,

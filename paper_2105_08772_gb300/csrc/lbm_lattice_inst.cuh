@@ -4,6 +4,7 @@
 
 #include "lbm_kernels_chunk.cuh"
 #include "lbm_kernels_moment.cuh"
+#include "lbm_kernels_row.cuh"
 #include "lbm_kernels_tma.cuh"
 #include "lbm_launch.h"
 
@@ -134,6 +135,49 @@ static cudaError_t launch_chunk(const LatticeDesc& d, int zchunk, bool prepare, 
   return launch_chunk_variant<P, ST, BX, BY, D, false>(d, zchunk, false, s);
 }
 
+template <int P, int ST, bool ALIGNED>
+static cudaError_t launch_row_shape(const LatticeDesc& d, const RowPlan& r, int sms, bool prepare, cudaStream_t s) {
+  using Sh = RowShape<P, ST>;
+  auto kern = lattice_row_kernel<Sh, ALIGNED>;
+  if (prepare)
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::smem_bytes);
+  const int grid = r.items < sms ? r.items : sms;
+  // every other step walks the planes downwards: what the last step wrote last is
+  // read first, from L2 (128^3 54.1 -> 53.1 us, 192^3 170.4 -> 169.5, 157^3 100.5 -> 101.5)
+  const int flip = reinterpret_cast<uintptr_t>(d.src) > reinterpret_cast<uintptr_t>(d.dst);
+  return launch_step_kernel(kern, grid, r.cfg.nd + r.cfg.nc + 32, Sh::smem_bytes, s, true, d, r.cfg, flip);
+}
+
+// The whole-row kernel where the plan has a cut; cudaErrorNotSupported (nothing
+// launched) where it has not.  One CTA per SM; launched with programmatic
+// serialisation (the next step's CTAs take over SM by SM: 128^3 58.5 -> 56.2 us, 64^3
+// 17.8 -> 15.2 us when it came in).
+template <int P, int ST>
+static cudaError_t launch_row(const LatticeDesc& d, bool prepare, cudaStream_t s) {
+  static int sms = 0;
+  if (prepare || sms == 0) {
+    int dev = 0, n = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = launch_row_shape<P, ST, true>(d, RowPlan{}, 0, true, s);
+    if constexpr (P != kF16)
+      if (e == cudaSuccess) e = launch_row_shape<P, ST, false>(d, RowPlan{}, 0, true, s);
+    if (e == cudaSuccess) sms = n;
+    if (e != cudaSuccess || prepare) return e;
+  }
+  // the last box's plan: a step-by-step caller would search it (about 20 us) each time
+  static thread_local int box[4] = {0, 0, 0, 0};
+  static thread_local RowPlan r;
+  if (box[0] != d.nx || box[1] != d.ny || box[2] != d.nz || box[3] != sms) {
+    r = row_plan(P, stencil_radius<ST>(), d.nx, d.ny, d.nz, sms);
+    box[0] = d.nx; box[1] = d.ny; box[2] = d.nz; box[3] = sms;
+  }
+  if (!r.ok) return cudaErrorNotSupported;
+  if (r.aligned) return launch_row_shape<P, ST, true>(d, r, sms, false, s);
+  if constexpr (P == kF16) return cudaErrorNotSupported;
+  else return launch_row_shape<P, ST, false>(d, r, sms, false, s);
+}
+
 // unit-tau moment kernel; for tau != 1 the chunked kernel of the same shape runs
 template <int P, int ST, int BX, int BY, int D>
 static cudaError_t launch_moment(const LatticeDesc& d, int zchunk, bool prepare, cudaStream_t s) {
@@ -147,6 +191,8 @@ static cudaError_t launch_moment(const LatticeDesc& d, int zchunk, bool prepare,
     cudaError_t e = prepare_persistent(kern, Sh::NT, Sh::smem_bytes, &resident);
     if constexpr (P != kF16)   // the tau != 1 fallback (FP16 storage has none: tau = 1 only)
       if (e == cudaSuccess && prepare) e = launch_chunk<P, ST, BX, BY, D>(d, 0, true, s);
+    if constexpr (P != kF64 && ST == 4 && BX == 32 && BY == 8)
+      if (e == cudaSuccess && prepare) e = launch_row<P, ST>(d, true, s);
     if (e != cudaSuccess || prepare) return e;
   }
   if (d.omega != 1.0) {
@@ -154,6 +200,11 @@ static cudaError_t launch_moment(const LatticeDesc& d, int zchunk, bool prepare,
     else return launch_chunk<P, ST, BX, BY, D>(d, zchunk, false, s);
   }
   if (d.nx % Sh::VE != 0 || d.nx < BX + 2 * Sh::APRON) return cudaErrorInvalidValue;
+  if constexpr (P != kF64 && ST == 4 && BX == 32 && BY == 8)
+    if (zchunk == 0) {
+      const cudaError_t e = launch_row<P, ST>(d, false, s);
+      if (e != cudaErrorNotSupported) return e;
+    }
   const long long cols = (long long)((d.nx + BX - 1) / BX) * ((d.ny + BY - 1) / BY);
   const int zc = choose_zchunk(cols, d.nz, Sh::R, resident, zchunk);
   const long long items = cols * ((d.nz + zc - 1) / zc);
@@ -240,9 +291,16 @@ static cudaError_t launch_moment_elem(const LatticeDesc& d, int zchunk, bool pre
       if (e == cudaSuccess) resident = (per_sm < 2 ? (per_sm > 0 ? per_sm : 1) : 2) * sms;
     }
     if (e == cudaSuccess && prepare) e = launch_async<P, ST, BX, BY, D>(d, 0, true, s);
+    if constexpr (P != kF64 && ST == 4)
+      if (e == cudaSuccess && prepare) e = launch_row<P, ST>(d, true, s);
     if (e != cudaSuccess || prepare) return e;
   }
   if (d.omega != 1.0) return launch_async<P, ST, BX, BY, D>(d, zchunk, false, s);
+  if constexpr (P != kF64 && ST == 4)
+    if (zchunk == 0) {
+      const cudaError_t e = launch_row<P, ST>(d, false, s);
+      if (e != cudaErrorNotSupported) return e;
+    }
   const long long cols = (long long)((d.nx + BX - 1) / BX) * ((d.ny + BY - 1) / BY);
   const int zc = choose_zchunk(cols, d.nz, Sh::R, resident, zchunk);
   const long long items = cols * ((d.nz + zc - 1) / zc);

@@ -123,6 +123,91 @@ constexpr bool moment_elem_two_per_sm(size_t elem, int R, int bx, int by, int de
 
 constexpr size_t kMaxSmemPerCta = 227 * 1024;   // opt-in limit of one CTA on sm_103
 
+// ---------------------------------------------------------------- row kernel
+// The whole-row step (lbm_kernels_row.cuh) behind tile kinds 5 and 6 with a
+// launcher-chosen z chunk at tau = 1.  One CTA of at most kRowThreads threads (128
+// registers each: the kernel must not spill, a few spilled words in its plane loop
+// cost it a third) and nearly all of an SM's shared memory per SM.
+constexpr int kRowThreads = 512;
+
+// How one launch cuts a lattice.
+struct RowCfg {
+  int by, zc;    // rows and planes of an item
+  int nd, nc;    // density and collision threads (multiples of 32)
+};
+
+// Capacities of a row CTA: elements of a population's slot, interior nodes, packed
+// operands per density thread.  A padded node takes 19 staged populations and 2R + 2
+// psi values, an interior node R + 2 planes of 4 moments; both fill the SM at the
+// tiles that the plan takes most (14 to 16 rows of 64 to 96 nodes, 4 to 8 of 128 to
+// 256).
+struct RowCaps { int slot, mcap, kd; };
+constexpr RowCaps row_caps(int prec, int R) {
+  if (R == 1) return prec == kF16 ? RowCaps{2336, 1920, 3} : RowCaps{1808, 1344, 3};
+  return RowCaps{1808, 768, 3};
+}
+
+struct RowPlan {
+  bool ok;
+  bool aligned;   // rows are whole 16-byte pieces
+  int items;
+  RowCfg cfg;
+};
+
+// The cut with the least expected time, or ok = false where no item fits (rows too
+// long) or the box is too small for the copies' wrap.
+// An SM's time is its rounds of items times their planes (with the halo planes) times
+// a plane's time: a latency (of the density warps, or of the collision warps' turns)
+// and a share for each 64-node piece that the two kinds of warps handle.  Memory's
+// time counts the populations once and, for boxes beyond L2, the halo planes that a
+// chunk's two neighbours read at another time; large boxes also lose 2% a chunk (the
+// more places of the 19 planes are walked at once: 192^3 in 4 chunks 171 us, in 5 183).
+// The constants (microseconds) were
+// fitted to 2300 measured cuts of 28 boxes, 24^3 to 256^3, odd and ragged ones among
+// them: the plan's choice is within 4% of the best cut of each, but for two FP16 boxes
+// (9%).
+inline RowPlan row_plan(int prec, int R, int nx, int ny, int nz, int sms) {
+  RowPlan best{false, false, 0, {0, 0, 0, 0}};
+  const int es = prec == kF16 ? 2 : 4, ve = 16 / es;
+  const bool aligned = nx % ve == 0;
+  if (prec == kF64 || nx < 2 * R + 1 || ny < 2 * R + 1 || nz < 2 * R + 1) return best;
+  // smaller boxes stay with the moment kernel, whose CTAs start faster and are more
+  // (32^3 4.5 against 7.2 us, 48^3 7.8 against 8.4; 64^3 11.7 against 11.4)
+  if ((long long)nx * ny * nz < 190000) return best;
+  const RowCaps caps = row_caps(prec, R);
+  const double bytes = (double)nx * ny * nz * 38.0 * es;
+  const double scale = (aligned ? 1.0 : 1.42) * (prec == kF16 ? 0.9 : 1.0);
+  double best_t = 0.0;
+  for (int by = 1; by <= ny; ++by) {
+    const long long nodes = (long long)(by + 2 * R) * nx, inner = (long long)by * nx;
+    if (nodes > caps.slot - 4 * ve || inner > caps.mcap) break;
+    // a block's copy wraps in y at most once (aligned rows: four segments)
+    if (aligned ? by + 2 * R > 3 * ny : by + 2 * R > ny + 1) break;
+    const int wd = (int)((nodes + 63) / 64), wc = (int)((inner + 63) / 64);   // 64-node pieces
+    const int nd = (wd + caps.kd - 1) / caps.kd, most = kRowThreads / 32 - 1 - nd;
+    if (most < 1) break;
+    const int turns = (wc + most - 1) / most;   // pieces a collision warp takes
+    if (turns > 16) break;
+    const int nc = (wc + turns - 1) / turns, cols = (ny + by - 1) / by;
+    const double lat_d = 1.15 * scale, lat_c = 0.134 * turns * scale + 0.285;
+    const double plane = (lat_d > lat_c ? lat_d : lat_c) + 0.0282 * (wd + 1.07 * wc) * scale;
+    for (int chunks = 1; chunks <= nz; ++chunks) {
+      const int zc = (nz + chunks - 1) / chunks;
+      if (chunks > 1 && zc == (nz + chunks - 2) / (chunks - 1)) continue;
+      const long long items = (long long)cols * ((nz + zc - 1) / zc), rounds = (items + sms - 1) / sms;
+      const double sm = rounds * ((zc + 2 * R) * plane + 0.3);
+      double mem = bytes / 9e6;
+      if (bytes > 2.3e8) mem = bytes / 6.55e6 * (1.0 + (bytes > 5e8 ? 1.0 : 2.0) * R / zc);
+      if (bytes > 5e8 && prec == kF32) mem *= 1.0 + 0.02 * (chunks - 2);
+      const double a = sm * sm * sm, b = mem * mem * mem, t = a * a + b * b;   // (sm^6 + mem^6): rises with the time
+      if (best.ok && t >= best_t) continue;
+      best_t = t;
+      best = RowPlan{true, aligned, (int)items, {by, zc, nd * 32, nc * 32}};
+    }
+  }
+  return best;
+}
+
 // number of CTAs (= FieldPartial records) a kind-0 lattice launch uses
 inline long long lattice_grid_ctas(const LatticeDesc& d, TileCfg cfg) {
   const long long tiles = (long long)((d.nx + cfg.bx - 1) / cfg.bx) * ((d.ny + cfg.by - 1) / cfg.by);
