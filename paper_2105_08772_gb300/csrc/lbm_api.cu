@@ -1398,6 +1398,7 @@ struct lbm_batch {
   cudaGraphExec_t graph = nullptr;
   int graph_len = 0;
   int graph_mode = -1;       // BatchMode the graph (and the table's tiling) was made for
+  int grid = 0;              // resident CTAs of that mode's kernel
   long long lattice_updates = 0;
   // configuration chosen by lbm_batch_autotune (defaults: the natural kernel mode,
   // z chunks of min(16, nz), every slot)
@@ -1445,7 +1446,10 @@ int natural_batch_mode(const lbm_batch* b);
 
 // the kernel modes that can run the whole queue, fastest first by construction
 std::vector<int> batch_modes_allowed(int natural, int prec) {
-  if (prec == kF16) return {kBatchMoment};   // the only FP16 batch kernel
+  if (prec == kF16) return natural == kBatchRow ? std::vector<int>{kBatchRow, kBatchMoment}
+                                                : std::vector<int>{kBatchMoment};
+  if (natural == kBatchRow) return {kBatchRow, kBatchMoment, kBatchUnitTau};
+  if (natural == kBatchRowAny) return {kBatchRowAny, kBatchMomentElem, kBatchUnitTau};
   if (natural == kBatchMoment) return {kBatchMoment, kBatchMomentElem, kBatchUnitTau};
   if (natural == kBatchMomentElem) return {kBatchMomentElem, kBatchUnitTau};
   return {natural};
@@ -1459,14 +1463,32 @@ int batch_mode(const lbm_batch* b) {
   return natural;
 }
 
-int natural_batch_mode(const lbm_batch* b) {
-  bool unit = true, moment = true;
-  const int bx = batch_tile(b->prec, b->stencil, kBatchMoment).bx;
-  for (const BatchRun& r : b->runs) {
-    if (r.tau != 1.0) unit = false;
-    if (r.box.nx % 4 != 0 || r.box.nx < bx + 8) moment = false;
+// The mode of a set of lattices: the row kernel where it takes every box and the
+// lattices together are worth its few large items (a launch of 152 CTAs; below
+// 190000 nodes in all the tile kernels' many small CTAs are faster, as for one lattice).
+struct BatchMix {
+  int prec, stencil;
+  bool unit = true, moment = true, aligned = true, rows = true;
+  double nodes = 0.0;
+  void add(lbm_box box, double tau) {
+    const int bx = batch_tile(prec, stencil, kBatchMoment).bx;
+    if (tau != 1.0) unit = false;
+    if (box.nx % 4 != 0 || box.nx < bx + 8) moment = false;
+    if (box.nx % (prec == kF16 ? 8 : 4) != 0) aligned = false;
+    if (row_batch_rows(prec, stencil, box.nx, box.ny, box.nz) == 0) rows = false;
+    nodes += (double)box.nx * box.ny * box.nz;
   }
-  return !unit ? kBatchMixedTau : (moment ? kBatchMoment : kBatchMomentElem);
+  int mode() const {
+    if (!unit) return kBatchMixedTau;
+    if (rows && nodes >= 190000.0) return aligned ? kBatchRow : kBatchRowAny;
+    return moment ? kBatchMoment : kBatchMomentElem;
+  }
+};
+
+int natural_batch_mode(const lbm_batch* b) {
+  BatchMix m{b->prec, b->stencil};
+  for (const BatchRun& r : b->runs) m.add(r.box, r.tau);
+  return m.mode();
 }
 
 lbm_status batch_fill(lbm_batch* b) {
@@ -1506,22 +1528,45 @@ lbm_status batch_fill(lbm_batch* b) {
   return LBM_OK;
 }
 
+// One z chunk for all lattices of a launch on `grid` resident CTAs, chosen like the
+// single-lattice launcher's (fewest rounds x planes).
+int common_zchunk(int prec, int stencil, int mode, const std::vector<lbm_ctx*>& ctx, int grid) {
+  const int R = radius_of(stencil);
+  int max_nz = 1, rows = 0;
+  for (const lbm_ctx* c : ctx)
+    if (c && c->box.nz > max_nz) max_nz = c->box.nz;
+  int best_zc = max_nz;
+  long long best_cost = -1;
+  for (int zc = 1; zc <= max_nz; ++zc) {
+    long long items = 0;
+    for (const lbm_ctx* c : ctx)
+      if (c) items += batch_items(prec, stencil, mode, c->box.nx, c->box.ny, c->box.nz, zc, &rows);
+    const long long rounds = (items + grid - 1) / grid, cost = rounds * (zc + 2 * R);
+    if (best_cost < 0 || cost <= best_cost) {
+      best_cost = cost;
+      best_zc = zc;
+    }
+  }
+  return best_zc;
+}
+
 // table of the active lattices, in slot order, with their global work items
 lbm_status batch_upload(lbm_batch* b) {
-  const TileCfg t = batch_tile(b->prec, b->stencil, b->graph_mode);
   b->table_host.clear();
   long long items = 0;
+  // tile kernels: chunks of 16 planes; the row kernel's few large items are evened out
+  const int auto_zc = batch_mode_row(b->graph_mode) && b->zchunk == 0 && b->grid > 0
+                          ? common_zchunk(b->prec, b->stencil, b->graph_mode, b->slot_ctx, b->grid) : 16;
   for (int k = 0; k < b->slots; ++k) {
     lbm_ctx* c = b->slot_ctx[k];
     if (!c) continue;
     BatchEntry e;
     e.d = desc_of(c, 0);
     e.parity = c->cur;
-    const int zc = b->zchunk > 0 ? b->zchunk : 16;
+    const int zc = b->zchunk > 0 ? b->zchunk : auto_zc;
     e.zchunk = c->box.nz < zc ? c->box.nz : zc;
     e.item_begin = items;
-    items += (long long)((c->box.nx + t.bx - 1) / t.bx) * ((c->box.ny + t.by - 1) / t.by) *
-             ((c->box.nz + e.zchunk - 1) / e.zchunk);
+    items += batch_items(b->prec, b->stencil, b->graph_mode, c->box.nx, c->box.ny, c->box.nz, e.zchunk, &e.rows);
     b->table_host.push_back(e);
   }
   b->hdr_host.n = (int)b->table_host.size();
@@ -1540,8 +1585,7 @@ lbm_status batch_graph(lbm_batch* b, int len, int mode) {
   if (b->graph && b->graph_len == len && b->graph_mode == mode) return LBM_OK;
   if (b->graph) cudaGraphExecDestroy(b->graph);
   b->graph = nullptr;
-  int grid = 0;
-  LBM_BCUDA(b, launch_batch(b->prec, b->stencil, mode, b->table_dev, b->hdr_dev, 0, true, &grid,
+  LBM_BCUDA(b, launch_batch(b->prec, b->stencil, mode, b->table_dev, b->hdr_dev, 0, true, &b->grid,
                                  b->stream));
   cudaGraph_t g = nullptr;
   LBM_BCUDA(b, cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal));
@@ -1801,7 +1845,9 @@ lbm_status lbm_batch_autotune(lbm_batch* b, int reps, long long* choice) {
   if (b->graph) cudaGraphExecDestroy(b->graph);
   b->graph = nullptr;
   b->graph_mode = -1;
-  if (choice) *choice = (long long)best_mode * 1000000 + (long long)best_zc * 1000 + best_cap;
+  // (the row kernel reports as the moment kernel that it stands in for)
+  const int shown = best_mode == kBatchRow ? kBatchMoment : (best_mode == kBatchRowAny ? kBatchMomentElem : best_mode);
+  if (choice) *choice = (long long)shown * 1000000 + (long long)best_zc * 1000 + best_cap;
   return LBM_OK;
 }
 
@@ -1856,24 +1902,7 @@ lbm_status gfail(lbm_group* g, lbm_status s, const char* fmt, ...) {
 // the table of the group's lattices with their current parities; one z chunk for
 // all of them, chosen like the single-lattice launcher (fewest rounds x planes)
 lbm_status group_upload(lbm_group* g) {
-  const TileCfg t = batch_tile(g->prec, g->stencil, g->mode);
-  const int R = radius_of(g->stencil);
-  int max_nz = 1;
-  for (lbm_ctx* c : g->ctx) max_nz = c->box.nz > max_nz ? c->box.nz : max_nz;
-  int best_zc = max_nz;
-  long long best_cost = -1;
-  for (int zc = 1; zc <= max_nz; ++zc) {
-    long long items = 0;
-    for (lbm_ctx* c : g->ctx)
-      items += (long long)((c->box.nx + t.bx - 1) / t.bx) * ((c->box.ny + t.by - 1) / t.by) *
-               ((c->box.nz + zc - 1) / zc);
-    const long long rounds = (items + g->grid - 1) / g->grid;
-    const long long cost = rounds * (zc + 2 * R);
-    if (best_cost < 0 || cost <= best_cost) {
-      best_cost = cost;
-      best_zc = zc;
-    }
-  }
+  const int best_zc = common_zchunk(g->prec, g->stencil, g->mode, g->ctx, g->grid);
   g->table_host.clear();
   long long items = 0;
   for (lbm_ctx* c : g->ctx) {
@@ -1882,8 +1911,7 @@ lbm_status group_upload(lbm_group* g) {
     e.parity = c->cur;
     e.zchunk = best_zc < c->box.nz ? best_zc : c->box.nz;
     e.item_begin = items;
-    items += (long long)((c->box.nx + t.bx - 1) / t.bx) * ((c->box.ny + t.by - 1) / t.by) *
-             ((c->box.nz + e.zchunk - 1) / e.zchunk);
+    items += batch_items(g->prec, g->stencil, g->mode, c->box.nx, c->box.ny, c->box.nz, e.zchunk, &e.rows);
     g->table_host.push_back(e);
   }
   g->hdr_host.n = (int)g->table_host.size();
@@ -1928,14 +1956,9 @@ lbm_status lbm_group_create(lbm_ctx* const* ctxs, int n, void* dev_workspace, si
   char* ws = static_cast<char*>(dev_workspace);
   g->table_dev = reinterpret_cast<BatchEntry*>(ws);
   g->hdr_dev = reinterpret_cast<BatchHeader*>(ws + align256(sizeof(BatchEntry) * (size_t)n));
-  // kernel mode as for a batch: the moment kernel when every lattice allows it
-  bool unit = true, moment = true;
-  const int bx = batch_tile(g->prec, g->stencil, kBatchMoment).bx;
-  for (lbm_ctx* c : g->ctx) {
-    if (c->tau != 1.0) unit = false;
-    if (c->box.nx % 4 != 0 || c->box.nx < bx + 8) moment = false;
-  }
-  g->mode = !unit ? kBatchMixedTau : (moment ? kBatchMoment : kBatchMomentElem);
+  BatchMix mix{g->prec, g->stencil};   // kernel mode as for a batch
+  for (lbm_ctx* c : g->ctx) mix.add(c->box, c->tau);
+  g->mode = mix.mode();
   cudaError_t e = cudaStreamCreateWithFlags(&g->cap_stream, cudaStreamNonBlocking);
   if (e == cudaSuccess)
     e = launch_batch(g->prec, g->stencil, g->mode, g->table_dev, g->hdr_dev, 0, true, &g->grid, g->stream);

@@ -222,6 +222,7 @@ struct BatchEntry {
   long long item_begin;
   int zchunk;
   int parity;
+  int rows;              // rows of an item (row kernel; 0: the tile kernels' tiles)
 };
 struct BatchHeader {
   int n;                 // active entries

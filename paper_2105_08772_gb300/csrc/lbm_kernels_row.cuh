@@ -591,4 +591,40 @@ __global__ void __launch_bounds__(kRowThreads, 1) lattice_row_kernel(LatticeDesc
   row_finish(smem_raw, c, uses, d.err);
 }
 
+// A batch of tau = 1 lattices (see lattice_async_batch_kernel for the table; here
+// every entry has its rows per item in `rows`).
+template <class Sh, bool ALIGNED>
+__global__ void __launch_bounds__(kRowThreads, 1)
+lattice_row_batch_kernel(const BatchEntry* __restrict__ table, const BatchHeader* __restrict__ hdr, int step) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  RowCfg c{0, 0, kRowBatchDensityWarps * 32, (int)blockDim.x - (kRowBatchDensityWarps + 1) * 32};
+  row_init(smem_raw, c);
+  step_grid_enter();
+  __syncthreads();
+  const int n = hdr->n;
+  const long long total = hdr->total_items;
+  unsigned uses = 0;
+#pragma unroll 1
+  for (long long item = blockIdx.x; item < total; item += gridDim.x) {
+    int lo = 0, hi = n - 1;          // last entry with item_begin <= item
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) / 2;
+      if (table[mid].item_begin <= item) lo = mid; else hi = mid - 1;
+    }
+    LatticeDesc d = table[lo].d;
+    if ((table[lo].parity ^ step) & 1) {
+      const void* t = d.src;
+      d.src = d.dst;
+      d.dst = const_cast<void*>(t);
+    }
+    c.by = table[lo].rows;
+    c.zc = table[lo].zchunk;
+    row_process_item<Sh, ALIGNED>(d, c, (int)(item - table[lo].item_begin), false, smem_raw, uses);
+    if (*reinterpret_cast<volatile int*>(smem_raw + kRowDead)) {   // this and every later item of the CTA
+      if (d.err) *reinterpret_cast<volatile int*>(d.err) = 1;
+    }
+  }
+  row_finish(smem_raw, c, uses, nullptr);
+}
+
 }  // namespace lbm

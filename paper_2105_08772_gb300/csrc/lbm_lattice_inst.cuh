@@ -388,16 +388,39 @@ static cudaError_t launch_moment_batch_variant(const BatchEntry* table, const Ba
   return launch_step_kernel(kern, resident, Sh::NT, Sh::smem_bytes, s, false, table, hdr, step);
 }
 
+template <int P, int ST, bool ALIGNED>
+static cudaError_t launch_row_batch(const BatchEntry* table, const BatchHeader* hdr, int step, bool prepare,
+                                    int* grid, cudaStream_t s) {
+  using Sh = RowShape<P, ST>;
+  auto kern = lattice_row_batch_kernel<Sh, ALIGNED>;
+  static int sms = 0;
+  if (prepare || sms == 0) {
+    int dev = 0, n = 0;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::smem_bytes);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    sms = n;
+  }
+  if (grid) *grid = sms;
+  if (prepare) return cudaSuccess;
+  return launch_step_kernel(kern, sms, (1 + kRowBatchDensityWarps + kRowBatchCollideWarps) * 32, Sh::smem_bytes, s,
+                            true, table, hdr, step);
+}
+
 // batches: the moment kernel when every lattice allows it, else the pipelined
 // kernel; 32 x 8 tiles for FP32 E4, 32 x 4 otherwise (batch_tile)
 template <int P, int ST>
 static cudaError_t dispatch_batch(int mode, const BatchEntry* table, const BatchHeader* hdr,
                                   int step, bool prepare, int* grid, cudaStream_t s) {
   if constexpr (P == kF16) {   // FP16 storage: the moment kernel, E4, 32 x 8 tiles
+    if (ST == 4 && mode == kBatchRow) return launch_row_batch<P, 4, true>(table, hdr, step, prepare, grid, s);
     if (ST == 4 && mode == kBatchMoment)
       return launch_moment_batch_variant<P, 4, 32, 8, 1>(table, hdr, step, prepare, grid, s);
     return cudaErrorInvalidValue;
   } else if constexpr (P == kF32 && ST == 4) {
+    if (mode == kBatchRow) return launch_row_batch<P, ST, true>(table, hdr, step, prepare, grid, s);
+    if (mode == kBatchRowAny) return launch_row_batch<P, ST, false>(table, hdr, step, prepare, grid, s);
     if (mode == kBatchMoment) return launch_moment_batch_variant<P, ST, 32, 8, 1>(table, hdr, step, prepare, grid, s);
     if (mode == kBatchMomentElem)
       return launch_moment_batch_variant<P, ST, 32, 8, 1, true>(table, hdr, step, prepare, grid, s);

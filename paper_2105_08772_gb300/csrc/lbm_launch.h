@@ -223,11 +223,44 @@ struct BatchHeader;
 // boxes the moment kernel takes (nx % 4 == 0, nx >= tile width + 8)
 // (kBatchMomentElem: all tau = 1, some box not split into 16-byte row chunks: the
 // moment kernel with element copies)
-enum BatchMode : int { kBatchMixedTau = 0, kBatchUnitTau = 1, kBatchMoment = 2, kBatchMomentElem = 3 };
+// (kBatchRow / kBatchRowAny: the row kernel, all boxes with aligned rows / any)
+enum BatchMode : int { kBatchMixedTau = 0, kBatchUnitTau = 1, kBatchMoment = 2, kBatchMomentElem = 3,
+                       kBatchRow = 4, kBatchRowAny = 5 };
+constexpr bool batch_mode_row(int mode) { return mode == kBatchRow || mode == kBatchRowAny; }
+// rows of a batch item of this box under the row kernel: as many as a CTA holds (all
+// items of a launch share one split of the warps), evened out over the box; 0 where
+// the row kernel does not take the box (or the storage or stencil)
+constexpr int kRowBatchDensityWarps = 9, kRowBatchCollideWarps = 6;
+inline int row_batch_rows(int prec, int stencil, int nx, int ny, int nz) {
+  if (stencil != 4 || prec == kF64 || nx < 3 || ny < 3 || nz < 3) return 0;
+  const RowCaps caps = row_caps(prec, 1);
+  const int ve = prec == kF16 ? 8 : 4;
+  int most = (int)(((long long)kRowBatchDensityWarps * caps.kd * 64) / nx);
+  if ((caps.slot - 4 * ve) / nx < most) most = (caps.slot - 4 * ve) / nx;
+  most -= 2;
+  if (caps.mcap / nx < most) most = caps.mcap / nx;
+  if (ny - 1 < most) most = ny - 1;
+  if (most < 1 || (prec == kF16 && nx % ve != 0)) return 0;
+  const int cols = (ny + most - 1) / most;
+  return (ny + cols - 1) / cols;
+}
+// (tile kernels only; the row kernel's items are whole rows)
 inline TileCfg batch_tile(int prec, int stencil, int mode) {
   TileCfg t{32, (stencil == 4 && (prec != kF64 || mode == kBatchMomentElem)) ? 8 : 4, 0};
   t.kind = mode == kBatchMoment ? 5 : (mode == kBatchMomentElem ? 6 : 1);
   return t;
+}
+// items of one lattice in a batch launch of this mode, z chunks of zc planes; *rows as
+// for BatchEntry::rows
+inline long long batch_items(int prec, int stencil, int mode, int nx, int ny, int nz, int zc, int* rows) {
+  const long long chunks = (nz + zc - 1) / zc;
+  if (batch_mode_row(mode)) {
+    *rows = row_batch_rows(prec, stencil, nx, ny, nz);
+    return chunks * ((ny + *rows - 1) / *rows);
+  }
+  *rows = 0;
+  const TileCfg t = batch_tile(prec, stencil, mode);
+  return chunks * ((nx + t.bx - 1) / t.bx) * ((ny + t.by - 1) / t.by);
 }
 cudaError_t launch_batch_f64(int stencil, int mode, const BatchEntry* table, const BatchHeader* hdr,
                              int step, bool prepare, int* grid, cudaStream_t s);
