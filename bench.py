@@ -57,7 +57,7 @@ def measured_peak_gbs():
 
 
 KERNEL_SOURCES = ("lbm_common.cuh", "lbm_exptab.cuh", "lbm_math.cuh", "lbm_kernels.cuh", "lbm_kernels_async.cuh", "lbm_kernels_chunk.cuh",
-                  "lbm_kernels_moment.cuh", "lbm_kernels_tma.cuh", "lbm_kernels_row.cuh", "lbm_launch.h", "lbm_lattice_inst.cuh")
+                  "lbm_kernels_moment.cuh", "lbm_kernels_tma.cuh", "lbm_kernels_row.cuh", "lbm_kernels_split.cuh", "lbm_launch.h", "lbm_lattice_inst.cuh")
 
 
 PROFILE_STEMS = {7: "lattice_tma", 6: "lattice_moment_elem", 5: "lattice_moment"}

@@ -117,7 +117,8 @@ typedef struct {
 /* ---------------------------------------------------------------- set-up */
 
 /* Bytes of device workspace one lattice needs (two population buffers of
- * 19 planes, a velocity snapshot for delta u, reduction scratch).  Returns 0
+ * 19 planes, a velocity snapshot for delta u, reduction scratch, for F64 a plane
+ * of psi).  Returns 0
  * for invalid arguments. */
 size_t lbm_workspace_bytes(lbm_box box, int stencil, int prec);
 

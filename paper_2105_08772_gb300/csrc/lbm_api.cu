@@ -40,6 +40,7 @@ struct lbm_ctx {
   double* n_line;
   double* PT_line;
   double* PN_line;
+  void* aux;                  // FP64: psi between the two passes of a step
   int line_len;
   int cur;                    // buffer holding the current state
   long long steps;
@@ -119,7 +120,7 @@ constexpr size_t kStateObs = 128;
 static_assert(sizeof(PointOut) <= kStateDP, "PointOut overlaps dP_prev");
 
 struct Layout {
-  size_t pop, u_old, partials, state, lines, total;
+  size_t pop, u_old, partials, state, lines, aux, total;
   long long npart;
 };
 
@@ -133,7 +134,8 @@ Layout layout_of(lbm_box b, int prec) {
   // state block: PointOut at 0, dP_prev at kStateDP, the lbm_obs record at kStateObs
   L.state = align256(kStateObs + sizeof(lbm_obs));
   L.lines = align256(3 * sizeof(double) * (size_t)(b.nx / 2 + 1));
-  L.total = 2 * L.pop + L.u_old + L.partials + L.state + L.lines;
+  L.aux = prec == kF64 ? align256(N * sizeof(double)) : 0;
+  L.total = 2 * L.pop + L.u_old + L.partials + L.state + L.lines + L.aux;
   return L;
 }
 
@@ -163,6 +165,7 @@ LatticeDesc desc_of(const lbm_ctx* c, int src_buf) {
   d.eos.Rgas = c->eos.Rgas;
   d.eos.T = c->eos.T;
   d.err = c->err_dev;
+  d.aux = c->aux;
   d.tma = c->tma.ok ? &c->tma : nullptr;
   set_float_params(d);
   return d;
@@ -566,6 +569,8 @@ lbm_status lbm_create(lbm_box box, double tau, double G, lbm_eos eos, int stenci
   c->n_line = reinterpret_cast<double*>(p);
   c->PT_line = c->n_line + c->line_len;
   c->PN_line = c->PT_line + c->line_len;
+  p += L.lines;
+  c->aux = L.aux ? p : nullptr;
   c->cur = 0;
   c->n0 = 0.0;
   c->scale = 1.0;

@@ -5,6 +5,7 @@
 #include "lbm_kernels_chunk.cuh"
 #include "lbm_kernels_moment.cuh"
 #include "lbm_kernels_row.cuh"
+#include "lbm_kernels_split.cuh"
 #include "lbm_kernels_tma.cuh"
 #include "lbm_launch.h"
 
@@ -176,6 +177,19 @@ static cudaError_t launch_row(const LatticeDesc& d, bool prepare, cudaStream_t s
   if (r.aligned) return launch_row_shape<P, ST, true>(d, r, sms, false, s);
   if constexpr (P == kF16) return cudaErrorNotSupported;
   else return launch_row_shape<P, ST, false>(d, r, sms, false, s);
+}
+
+// The FP64 step in two passes.  Blocks of one warp while that leaves SMs without a
+// second one (their FP64 units work warp by warp), else of four.
+template <int ST>
+static cudaError_t launch_split(const LatticeDesc& d, cudaStream_t s) {
+  const long long warps = (d.plane + 31) / 32;
+  const int threads = warps <= 4096 ? 32 : 128;
+  const long long grid = (d.plane + threads - 1) / threads;
+  cudaError_t e = launch_step_kernel(split_moments_kernel, grid, threads, 0, s, false, d);
+  if (e != cudaSuccess) return e;
+  if (d.omega == 1.0) return launch_step_kernel(split_collide_kernel<ST, true>, grid, threads, 0, s, false, d);
+  return launch_step_kernel(split_collide_kernel<ST, false>, grid, threads, 0, s, false, d);
 }
 
 // unit-tau moment kernel; for tau != 1 the chunked kernel of the same shape runs
@@ -499,6 +513,14 @@ static cudaError_t dispatch_lattice(int stencil, int mode, const LatticeDesc& d,
   if (mode == kModeStep && c.kind == 7) {
     if (stencil == 4) return dispatch_tma<P, 4>(d, c, s);
     return cudaErrorInvalidValue;
+  }
+  if constexpr (P == kF64) {   // kinds 5 and 6 with a launcher-chosen z chunk: the two passes
+    if (mode == kModeStep && (c.kind == 5 || c.kind == 6) && c.zchunk == 0 && !c.prepare && d.aux) {
+      if (stencil == 4) return launch_split<4>(d, s);
+      if (stencil == 6) return launch_split<6>(d, s);
+      if (stencil == 8) return launch_split<8>(d, s);
+      return cudaErrorInvalidValue;
+    }
   }
   if (mode == kModeStep && c.kind == 6) {
     if (stencil == 4) return dispatch_moment_elem<P, 4>(d, c, s);
