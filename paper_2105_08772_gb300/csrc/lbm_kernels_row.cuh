@@ -592,17 +592,24 @@ __global__ void __launch_bounds__(kRowThreads, 1) lattice_row_kernel(LatticeDesc
 }
 
 // A batch of tau = 1 lattices (see lattice_async_batch_kernel for the table; here
-// every entry has its rows per item in `rows`).
+// every entry has its rows per item in `rows`).  Each role keeps its own copy of the
+// item's lattice in shared memory: in registers it would spill, and roles may be
+// at different items.
 template <class Sh, bool ALIGNED>
 __global__ void __launch_bounds__(kRowThreads, 1)
 lattice_row_batch_kernel(const BatchEntry* __restrict__ table, const BatchHeader* __restrict__ hdr, int step) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ LatticeDesc lattice[3];
   RowCfg c{0, 0, kRowBatchDensityWarps * 32, (int)blockDim.x - (kRowBatchDensityWarps + 1) * 32};
   row_init(smem_raw, c);
   step_grid_enter();
   __syncthreads();
   const int n = hdr->n;
   const long long total = hdr->total_items;
+  const int tid = threadIdx.x, role = tid < c.nd ? 0 : (tid < c.nd + c.nc ? 1 : 2);
+  const int first = role == 0 ? 0 : (role == 1 ? c.nd : c.nd + c.nc);
+  const int members = role == 0 ? c.nd : (role == 1 ? c.nc : 32);
+  LatticeDesc& d = lattice[role];
   unsigned uses = 0;
 #pragma unroll 1
   for (long long item = blockIdx.x; item < total; item += gridDim.x) {
@@ -611,15 +618,19 @@ lattice_row_batch_kernel(const BatchEntry* __restrict__ table, const BatchHeader
       const int mid = (lo + hi + 1) / 2;
       if (table[mid].item_begin <= item) lo = mid; else hi = mid - 1;
     }
-    LatticeDesc d = table[lo].d;
-    if ((table[lo].parity ^ step) & 1) {
-      const void* t = d.src;
-      d.src = d.dst;
-      d.dst = const_cast<void*>(t);
+    const BatchEntry& e = table[lo];
+    asm volatile("bar.sync %0, %1;\n" ::"r"(2 + role), "r"(members) : "memory");   // the role is done with the last one
+    if (tid == first) {
+      d = e.d;
+      if ((e.parity ^ step) & 1) {
+        d.src = e.d.dst;
+        d.dst = const_cast<void*>(e.d.src);
+      }
     }
-    c.by = table[lo].rows;
-    c.zc = table[lo].zchunk;
-    row_process_item<Sh, ALIGNED>(d, c, (int)(item - table[lo].item_begin), false, smem_raw, uses);
+    asm volatile("bar.sync %0, %1;\n" ::"r"(2 + role), "r"(members) : "memory");
+    c.by = e.rows;
+    c.zc = e.zchunk;
+    row_process_item<Sh, ALIGNED>(d, c, (int)(item - e.item_begin), false, smem_raw, uses);
     if (*reinterpret_cast<volatile int*>(smem_raw + kRowDead)) {   // this and every later item of the CTA
       if (d.err) *reinterpret_cast<volatile int*>(d.err) = 1;
     }
