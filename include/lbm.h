@@ -117,9 +117,8 @@ typedef struct {
 /* ---------------------------------------------------------------- set-up */
 
 /* Bytes of device workspace one lattice needs (two population buffers of
- * 19 planes, a velocity snapshot for delta u, reduction scratch, for F64 a plane
- * of psi).  Returns 0
- * for invalid arguments. */
+ * 19 planes, a velocity snapshot for delta u, reduction scratch, for F64 and
+ * F32 a plane of psi).  Returns 0 for invalid arguments. */
 size_t lbm_workspace_bytes(lbm_box box, int stencil, int prec);
 
 /* Create a context for one periodic lattice (Sec. II).  tau: BGK relaxation
@@ -236,8 +235,12 @@ lbm_status lbm_autotune(lbm_ctx* ctx, int reps, long long* choice);
  * and 5 need nx % 4 == 0 and nx >= bx + 8; 6 is compiled
  * for 32 x 8 tiles with E4 (depth 1, and depth 2 in F32) and 32 x 4 with E6/E8
  * (depth 1).  Kind 5 also takes F16 storage (E4, 32 x 8 tiles, tau = 1,
- * nx % 8 == 0, nx >= 48).  The default (lbm_create) is kind 5 where it applies,
- * else kind 6, else kind 1 (kind 5 or 0 for F16).  A code that is not compiled
+ * nx % 8 == 0, nx >= 48).  Kinds 5 and 6 with z chunk 0 stand for the fastest
+ * kernel of the box: the whole-row kernel (E4, tau = 1, F32 and F16, from some
+ * 200000 to 1200000 nodes on, rows of up to 597 / 768 nodes), the step in two passes
+ * (F64; F32 with E6 / E8, tau != 1 or smaller boxes), else the kernel of that name; with a z chunk
+ * given, always the kernel of that name.  The default (lbm_create) is kind 5 where it
+ * applies, else kind 6, else kind 1 (kind 5 or 0 for F16).  A code that is not compiled
  * for this context's precision, stencil and box gives LBM_EINVAL.  lbm_get_tile
  * returns the current code.  In F32/F64 storage results do not depend on the
  * choice: all kinds do the same arithmetic per node and give bitwise-equal
@@ -356,8 +359,9 @@ lbm_status lbm_batch_run(lbm_batch* b, long long max_steps, long long check_ever
 lbm_status lbm_batch_result(const lbm_batch* b, int id, lbm_obs* out);
 /* Batch autotuner: fills the slots from the queue, times `reps` (>= 2, rounded up
  * to even) launches of the batch step for every candidate -- kernel mode (the
- * row-chunk moment kernel, the element-copy moment kernel, the pipelined kernel,
- * where the queue allows each; F16: the moment kernel only), z chunk (8, 16, 32
+ * row-chunk moment kernel, the element-copy moment kernel -- with E4 the whole-row
+ * kernel behind both --, the pipelined kernel, where the queue allows each; F16: the
+ * first only), z chunk (8, 16, 32
  * planes) and slot count (all
  * slots, or half of them when at least four lattices are resident) -- and keeps
  * the one with the most lattice updates per second for lbm_batch_run.  The

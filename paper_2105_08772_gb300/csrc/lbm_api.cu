@@ -40,7 +40,7 @@ struct lbm_ctx {
   double* n_line;
   double* PT_line;
   double* PN_line;
-  void* aux;                  // FP64: psi between the two passes of a step
+  void* aux;                  // FP64, FP32: psi between the two passes of a step
   int line_len;
   int cur;                    // buffer holding the current state
   long long steps;
@@ -134,7 +134,7 @@ Layout layout_of(lbm_box b, int prec) {
   // state block: PointOut at 0, dP_prev at kStateDP, the lbm_obs record at kStateObs
   L.state = align256(kStateObs + sizeof(lbm_obs));
   L.lines = align256(3 * sizeof(double) * (size_t)(b.nx / 2 + 1));
-  L.aux = prec == kF64 ? align256(N * sizeof(double)) : 0;
+  L.aux = prec == kF16 ? 0 : align256(N * storage_bytes(prec));
   L.total = 2 * L.pop + L.u_old + L.partials + L.state + L.lines + L.aux;
   return L;
 }
@@ -1470,7 +1470,7 @@ int batch_mode(const lbm_batch* b) {
 
 // The mode of a set of lattices: the row kernel where it takes every box and the
 // lattices together are worth its few large items (a launch of 152 CTAs; below
-// 190000 nodes in all the tile kernels' many small CTAs are faster, as for one lattice).
+// 190000 nodes in all the tile kernels' many small CTAs are faster).
 struct BatchMix {
   int prec, stencil;
   bool unit = true, moment = true, aligned = true, rows = true;

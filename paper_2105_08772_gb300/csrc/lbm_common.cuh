@@ -140,7 +140,7 @@ struct LatticeDesc {
   EosParams eos;
   float n0f, omegaf, scalef, inv_scalef;   // n0, omega, scale, 1/scale rounded to float (host)
   int* err;             // device flag set by a kernel whose bounded wait ran out (may be null)
-  void* aux;            // FP64: one plane of psi between the two passes of a step (may be null)
+  void* aux;            // one plane of psi between the two passes of a step (null: FP16)
   const void* tma;      // host: the lattice's TMA tensor maps (TmaMaps) or null; kernels ignore it
 };
 

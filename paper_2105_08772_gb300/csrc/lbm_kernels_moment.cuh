@@ -1,6 +1,8 @@
-// Unit-relaxation-time variant of the pipelined Shan-Chen step (FP32 / FP64).  FP32 and
-// FP16 E4 boxes of 190000 nodes and more take the row kernel (lbm_kernels_row.cuh)
-// unless a z chunk is fixed; this one runs the rest.
+// Unit-relaxation-time variant of the pipelined Shan-Chen step.  Without a fixed z
+// chunk FP32 and FP64 boxes take the row kernel (lbm_kernels_row.cuh) or the two passes
+// (lbm_kernels_split.cuh) but for large FP32 boxes whose rows are too long for an item,
+// FP16 boxes below 190000 nodes are this kernel's; it also runs the batches that the
+// row batch kernel does not take.
 //
 // With tau = 1 the BGK update of Eq. (4) loses its f_i term:
 //     f*_i = f_i - (f_i - f_i^eq) + F_i = f_i^eq(n, u) + F_i,

@@ -64,7 +64,7 @@ struct RowShape {
   using T = typename Storage<P>::T;
   using S = typename Storage<P>::S;
   static constexpr int R = stencil_radius<ST>();
-  static constexpr RowCaps caps = row_caps(P, R);
+  static constexpr RowCaps caps = row_caps(P);
   static constexpr int SLOT = caps.slot;                   // elements of one population's slot
   static constexpr int MCAP = caps.mcap;                   // interior nodes of an item at most
   static constexpr int KD = caps.kd;                       // packed operands a density thread takes
@@ -91,11 +91,6 @@ template <> struct Pack<float> {
   using V = float2;
   static __device__ __forceinline__ float get(float2 v, int i) { return i == 0 ? v.x : v.y; }
   static __device__ __forceinline__ float2 make(float a, float b) { return make_float2(a, b); }
-};
-template <> struct Pack<double> {
-  using V = double;
-  static __device__ __forceinline__ double get(double v, int) { return v; }
-  static __device__ __forceinline__ double make(double a, double) { return a; }
 };
 
 __device__ __forceinline__ void row_bulk_copy(void* dst, const void* src, unsigned bytes, unsigned long long* bar) {
@@ -448,7 +443,7 @@ __device__ __forceinline__ void row_process_item(const LatticeDesc& d, const Row
   const int inner = h * nx;
   const long long pbytes = d.plane * (long long)sizeof(S);
   // which of the thread's nodes (unit u, node w: bit u PW + w) have wrapping x-neighbours
-  unsigned lm = 0, rm = 0, lm2 = 0, rm2 = 0;
+  unsigned lm = 0, rm = 0;
   {
     int u = 0;
     for (int f = N::first(tc); f < inner; f = N::first(tc + ++u * c.nc)) {
@@ -458,8 +453,6 @@ __device__ __forceinline__ void row_process_item(const LatticeDesc& d, const Row
         const unsigned bit = 1u << (u * PW + w);
         if (x == 0) lm |= bit;
         if (x == nx - 1) rm |= bit;
-        if (R == 2 && x < 2) lm2 |= bit;
-        if (R == 2 && x >= nx - 2) rm2 |= bit;
       }
     }
   }
@@ -486,37 +479,25 @@ __device__ __forceinline__ void row_process_item(const LatticeDesc& d, const Row
       const int f = N::first(tc + u * c.nc);
       if (f >= inner) break;
       const unsigned jc = (unsigned)(f * (int)sizeof(T));
-      // x-neighbours of node w at dx = -1, +1 (and -2, +2), bytes
-      unsigned xl[PW], xr[PW], xl2[R == 2 ? PW : 1], xr2[R == 2 ? PW : 1];
+      // x-neighbours of node w at dx = -1, +1, bytes
+      unsigned xl[PW], xr[PW];
 #pragma unroll
       for (int w = 0; w < PW; ++w) {
         const unsigned jw = jc + (unsigned)(w * N::NEXT * (int)sizeof(T)), bit = 1u << (u * PW + w);
         xl[w] = jw + ((lm & bit) ? lw : (unsigned)-(int)sizeof(T));
         xr[w] = jw + ((rm & bit) ? rw : (unsigned)sizeof(T));
-        if constexpr (R == 2) {
-          xl2[w] = jw + ((lm2 & bit) ? lw - (unsigned)sizeof(T) : (unsigned)(-2 * (int)sizeof(T)));
-          xr2[w] = jw + ((rm2 & bit) ? rw + (unsigned)sizeof(T) : (unsigned)(2 * (int)sizeof(T)));
-        }
       }
       auto at = [&](int dx, int dy, int dz) {
         const unsigned row = pl[dz + R][dy + R];
         if constexpr (N::PAIR) {
           if (dx == 0) return row_ld<V>(smem, row + jc);
-          if constexpr (R == 2) {
-            if (dx == 2) return row_ld<V>(smem, row + xr2[0]);
-            if (dx == -2) return row_ld<V>(smem, row + xl2[0]);
-          }
           if (dx < 0) return Pack<T>::make(row_ld<T>(smem, row + xl[0]), row_ld<T>(smem, row + jc));
           return Pack<T>::make(row_ld<T>(smem, row + jc + (unsigned)sizeof(T)), row_ld<T>(smem, row + xr[PW - 1]));
         } else {
           T v[2] = {(T)0, (T)0};
 #pragma unroll
           for (int w = 0; w < PW; ++w)
-            if constexpr (R == 2)
-              v[w] = row_ld<T>(smem, row + (dx == 0 ? jc + (unsigned)(w * N::NEXT * (int)sizeof(T))
-                                            : dx == 1 ? xr[w] : dx == -1 ? xl[w] : dx == 2 ? xr2[w] : xl2[w]));
-            else
-              v[w] = row_ld<T>(smem, row + (dx == 0 ? jc + (unsigned)(w * N::NEXT * (int)sizeof(T)) : dx > 0 ? xr[w] : xl[w]));
+            v[w] = row_ld<T>(smem, row + (dx == 0 ? jc + (unsigned)(w * N::NEXT * (int)sizeof(T)) : dx > 0 ? xr[w] : xl[w]));
           return Pack<T>::make(v[0], v[1]);
         }
       };

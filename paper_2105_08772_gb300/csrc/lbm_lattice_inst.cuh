@@ -4,10 +4,10 @@
 
 #include "lbm_kernels_chunk.cuh"
 #include "lbm_kernels_moment.cuh"
-#include "lbm_kernels_row.cuh"
 #include "lbm_kernels_split.cuh"
 #include "lbm_kernels_tma.cuh"
 #include "lbm_launch.h"
+#include "lbm_step_launch.h"
 
 namespace lbm {
 
@@ -43,30 +43,6 @@ inline int choose_zchunk(long long cols, int nz, int R, long long resident, int 
     }
   }
   return best_zc;
-}
-
-// Single-lattice step kernels whose CTAs take several work items in turn are
-// launched with programmatic stream serialisation (each kernel begins with
-// step_grid_enter): the next step's CTAs take the slots this step's CTAs free
-// and wait on the device for its completion, so consecutive steps' launch
-// latency and CTA ramp overlap the previous step's tail (256^3: 499 -> 488 us).
-// A grid of one item per CTA has no such tail and measured 0.6 us slower with it
-// (128^3), and the batch kernel measured 26% slower over a 144-lattice sweep, so
-// both are launched plainly.
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_step_kernel(void (*kern)(KArgs...), long long grid, int threads, size_t smem,
-                                      cudaStream_t s, bool overlap, Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
 template <typename Kern>
@@ -136,60 +112,21 @@ static cudaError_t launch_chunk(const LatticeDesc& d, int zchunk, bool prepare, 
   return launch_chunk_variant<P, ST, BX, BY, D, false>(d, zchunk, false, s);
 }
 
-template <int P, int ST, bool ALIGNED>
-static cudaError_t launch_row_shape(const LatticeDesc& d, const RowPlan& r, int sms, bool prepare, cudaStream_t s) {
-  using Sh = RowShape<P, ST>;
-  auto kern = lattice_row_kernel<Sh, ALIGNED>;
-  if (prepare)
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::smem_bytes);
-  const int grid = r.items < sms ? r.items : sms;
-  // every other step walks the planes downwards: what the last step wrote last is
-  // read first, from L2 (128^3 54.1 -> 53.1 us, 192^3 170.4 -> 169.5, 157^3 100.5 -> 101.5)
-  const int flip = reinterpret_cast<uintptr_t>(d.src) > reinterpret_cast<uintptr_t>(d.dst);
-  return launch_step_kernel(kern, grid, r.cfg.nd + r.cfg.nc + 32, Sh::smem_bytes, s, true, d, r.cfg, flip);
-}
+// the tile shapes whose launches with a launcher-chosen z chunk may take the row kernel
+template <int P, int ST, int BX, int BY>
+constexpr bool kRowKind = P != kF64 && ST == 4 && BX == 32 && BY == 8;
 
-// The whole-row kernel where the plan has a cut; cudaErrorNotSupported (nothing
-// launched) where it has not.  One CTA per SM; launched with programmatic
-// serialisation (the next step's CTAs take over SM by SM: 128^3 58.5 -> 56.2 us, 64^3
-// 17.8 -> 15.2 us when it came in).
-template <int P, int ST>
-static cudaError_t launch_row(const LatticeDesc& d, bool prepare, cudaStream_t s) {
-  static int sms = 0;
-  if (prepare || sms == 0) {
-    int dev = 0, n = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = launch_row_shape<P, ST, true>(d, RowPlan{}, 0, true, s);
-    if constexpr (P != kF16)
-      if (e == cudaSuccess) e = launch_row_shape<P, ST, false>(d, RowPlan{}, 0, true, s);
-    if (e == cudaSuccess) sms = n;
-    if (e != cudaSuccess || prepare) return e;
-  }
-  // the last box's plan: a step-by-step caller would search it (about 20 us) each time
-  static thread_local int box[4] = {0, 0, 0, 0};
-  static thread_local RowPlan r;
-  if (box[0] != d.nx || box[1] != d.ny || box[2] != d.nz || box[3] != sms) {
-    r = row_plan(P, stencil_radius<ST>(), d.nx, d.ny, d.nz, sms);
-    box[0] = d.nx; box[1] = d.ny; box[2] = d.nz; box[3] = sms;
-  }
-  if (!r.ok) return cudaErrorNotSupported;
-  if (r.aligned) return launch_row_shape<P, ST, true>(d, r, sms, false, s);
-  if constexpr (P == kF16) return cudaErrorNotSupported;
-  else return launch_row_shape<P, ST, false>(d, r, sms, false, s);
-}
-
-// The FP64 step in two passes.  Blocks of one warp while that leaves SMs without a
+// The step in two passes.  FP64: blocks of one warp while that leaves SMs without a
 // second one (their FP64 units work warp by warp), else of four.
-template <int ST>
+template <typename T, int ST>
 static cudaError_t launch_split(const LatticeDesc& d, cudaStream_t s) {
   const long long warps = (d.plane + 31) / 32;
-  const int threads = warps <= 4096 ? 32 : 128;
+  const int threads = sizeof(T) == 8 && warps <= 4096 ? 32 : 128;
   const long long grid = (d.plane + threads - 1) / threads;
-  cudaError_t e = launch_step_kernel(split_moments_kernel, grid, threads, 0, s, false, d);
+  cudaError_t e = launch_step_kernel(split_moments_kernel<T>, grid, threads, 0, s, false, d);
   if (e != cudaSuccess) return e;
-  if (d.omega == 1.0) return launch_step_kernel(split_collide_kernel<ST, true>, grid, threads, 0, s, false, d);
-  return launch_step_kernel(split_collide_kernel<ST, false>, grid, threads, 0, s, false, d);
+  if (d.omega == 1.0) return launch_step_kernel(split_collide_kernel<T, ST, true>, grid, threads, 0, s, false, d);
+  return launch_step_kernel(split_collide_kernel<T, ST, false>, grid, threads, 0, s, false, d);
 }
 
 // unit-tau moment kernel; for tau != 1 the chunked kernel of the same shape runs
@@ -205,8 +142,8 @@ static cudaError_t launch_moment(const LatticeDesc& d, int zchunk, bool prepare,
     cudaError_t e = prepare_persistent(kern, Sh::NT, Sh::smem_bytes, &resident);
     if constexpr (P != kF16)   // the tau != 1 fallback (FP16 storage has none: tau = 1 only)
       if (e == cudaSuccess && prepare) e = launch_chunk<P, ST, BX, BY, D>(d, 0, true, s);
-    if constexpr (P != kF64 && ST == 4 && BX == 32 && BY == 8)
-      if (e == cudaSuccess && prepare) e = launch_row<P, ST>(d, true, s);
+    if constexpr (kRowKind<P, ST, BX, BY>)
+      if (e == cudaSuccess && prepare) e = launch_row_any(P, d, true, s);
     if (e != cudaSuccess || prepare) return e;
   }
   if (d.omega != 1.0) {
@@ -214,11 +151,6 @@ static cudaError_t launch_moment(const LatticeDesc& d, int zchunk, bool prepare,
     else return launch_chunk<P, ST, BX, BY, D>(d, zchunk, false, s);
   }
   if (d.nx % Sh::VE != 0 || d.nx < BX + 2 * Sh::APRON) return cudaErrorInvalidValue;
-  if constexpr (P != kF64 && ST == 4 && BX == 32 && BY == 8)
-    if (zchunk == 0) {
-      const cudaError_t e = launch_row<P, ST>(d, false, s);
-      if (e != cudaErrorNotSupported) return e;
-    }
   const long long cols = (long long)((d.nx + BX - 1) / BX) * ((d.ny + BY - 1) / BY);
   const int zc = choose_zchunk(cols, d.nz, Sh::R, resident, zchunk);
   const long long items = cols * ((d.nz + zc - 1) / zc);
@@ -305,16 +237,11 @@ static cudaError_t launch_moment_elem(const LatticeDesc& d, int zchunk, bool pre
       if (e == cudaSuccess) resident = (per_sm < 2 ? (per_sm > 0 ? per_sm : 1) : 2) * sms;
     }
     if (e == cudaSuccess && prepare) e = launch_async<P, ST, BX, BY, D>(d, 0, true, s);
-    if constexpr (P != kF64 && ST == 4)
-      if (e == cudaSuccess && prepare) e = launch_row<P, ST>(d, true, s);
+    if constexpr (kRowKind<P, ST, BX, BY>)
+      if (e == cudaSuccess && prepare) e = launch_row_any(P, d, true, s);
     if (e != cudaSuccess || prepare) return e;
   }
   if (d.omega != 1.0) return launch_async<P, ST, BX, BY, D>(d, zchunk, false, s);
-  if constexpr (P != kF64 && ST == 4)
-    if (zchunk == 0) {
-      const cudaError_t e = launch_row<P, ST>(d, false, s);
-      if (e != cudaErrorNotSupported) return e;
-    }
   const long long cols = (long long)((d.nx + BX - 1) / BX) * ((d.ny + BY - 1) / BY);
   const int zc = choose_zchunk(cols, d.nz, Sh::R, resident, zchunk);
   const long long items = cols * ((d.nz + zc - 1) / zc);
@@ -402,39 +329,19 @@ static cudaError_t launch_moment_batch_variant(const BatchEntry* table, const Ba
   return launch_step_kernel(kern, resident, Sh::NT, Sh::smem_bytes, s, false, table, hdr, step);
 }
 
-template <int P, int ST, bool ALIGNED>
-static cudaError_t launch_row_batch(const BatchEntry* table, const BatchHeader* hdr, int step, bool prepare,
-                                    int* grid, cudaStream_t s) {
-  using Sh = RowShape<P, ST>;
-  auto kern = lattice_row_batch_kernel<Sh, ALIGNED>;
-  static int sms = 0;
-  if (prepare || sms == 0) {
-    int dev = 0, n = 0;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::smem_bytes);
-    if (e == cudaSuccess) e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    sms = n;
-  }
-  if (grid) *grid = sms;
-  if (prepare) return cudaSuccess;
-  return launch_step_kernel(kern, sms, (1 + kRowBatchDensityWarps + kRowBatchCollideWarps) * 32, Sh::smem_bytes, s,
-                            true, table, hdr, step);
-}
-
 // batches: the moment kernel when every lattice allows it, else the pipelined
 // kernel; 32 x 8 tiles for FP32 E4, 32 x 4 otherwise (batch_tile)
 template <int P, int ST>
 static cudaError_t dispatch_batch(int mode, const BatchEntry* table, const BatchHeader* hdr,
                                   int step, bool prepare, int* grid, cudaStream_t s) {
   if constexpr (P == kF16) {   // FP16 storage: the moment kernel, E4, 32 x 8 tiles
-    if (ST == 4 && mode == kBatchRow) return launch_row_batch<P, 4, true>(table, hdr, step, prepare, grid, s);
+    if (ST == 4 && mode == kBatchRow) return launch_row_batch_any(P, true, table, hdr, step, prepare, grid, s);
     if (ST == 4 && mode == kBatchMoment)
       return launch_moment_batch_variant<P, 4, 32, 8, 1>(table, hdr, step, prepare, grid, s);
     return cudaErrorInvalidValue;
   } else if constexpr (P == kF32 && ST == 4) {
-    if (mode == kBatchRow) return launch_row_batch<P, ST, true>(table, hdr, step, prepare, grid, s);
-    if (mode == kBatchRowAny) return launch_row_batch<P, ST, false>(table, hdr, step, prepare, grid, s);
+    if (mode == kBatchRow) return launch_row_batch_any(P, true, table, hdr, step, prepare, grid, s);
+    if (mode == kBatchRowAny) return launch_row_batch_any(P, false, table, hdr, step, prepare, grid, s);
     if (mode == kBatchMoment) return launch_moment_batch_variant<P, ST, 32, 8, 1>(table, hdr, step, prepare, grid, s);
     if (mode == kBatchMomentElem)
       return launch_moment_batch_variant<P, ST, 32, 8, 1, true>(table, hdr, step, prepare, grid, s);
@@ -514,12 +421,22 @@ static cudaError_t dispatch_lattice(int stencil, int mode, const LatticeDesc& d,
     if (stencil == 4) return dispatch_tma<P, 4>(d, c, s);
     return cudaErrorInvalidValue;
   }
-  if constexpr (P == kF64) {   // kinds 5 and 6 with a launcher-chosen z chunk: the two passes
-    if (mode == kModeStep && (c.kind == 5 || c.kind == 6) && c.zchunk == 0 && !c.prepare && d.aux) {
-      if (stencil == 4) return launch_split<4>(d, s);
-      if (stencil == 6) return launch_split<6>(d, s);
-      if (stencil == 8) return launch_split<8>(d, s);
-      return cudaErrorInvalidValue;
+  // kinds 5 and 6 with a launcher-chosen z chunk: the row kernel where it has a plan,
+  // the two passes where they are the fastest (split_applies)
+  if (mode == kModeStep && (c.kind == 5 || c.kind == 6) && c.zchunk == 0 && !c.prepare) {
+    if constexpr (P != kF64)
+      if (stencil == 4 && d.omega == 1.0 && c.bx == 32 && c.by == 8) {
+        const cudaError_t e = launch_row_any(P, d, false, s);
+        if (e != cudaErrorNotSupported) return e;
+      }
+    if constexpr (P != kF16) {
+      using T = typename Storage<P>::T;
+      if (d.aux && split_applies(P, stencil, d.omega == 1.0, d.plane)) {
+        if (stencil == 4) return launch_split<T, 4>(d, s);
+        if (stencil == 6) return launch_split<T, 6>(d, s);
+        if (stencil == 8) return launch_split<T, 8>(d, s);
+        return cudaErrorInvalidValue;
+      }
     }
   }
   if (mode == kModeStep && c.kind == 6) {

@@ -138,13 +138,21 @@ struct RowCfg {
 
 // Capacities of a row CTA: elements of a population's slot, interior nodes, packed
 // operands per density thread.  A padded node takes 19 staged populations and 2R + 2
-// psi values, an interior node R + 2 planes of 4 moments; both fill the SM at the
+// psi values, an interior node R + 2 planes of 4 moments (R = 1); both fill the SM at the
 // tiles that the plan takes most (14 to 16 rows of 64 to 96 nodes, 4 to 8 of 128 to
 // 256).
 struct RowCaps { int slot, mcap, kd; };
-constexpr RowCaps row_caps(int prec, int R) {
-  if (R == 1) return prec == kF16 ? RowCaps{2336, 1920, 3} : RowCaps{1808, 1344, 3};
-  return RowCaps{1808, 768, 3};
+constexpr RowCaps row_caps(int prec) {
+  return prec == kF16 ? RowCaps{2336, 1920, 3} : RowCaps{1808, 1344, 3};
+}
+
+// Smaller boxes have no row plan: the two passes (F32) and the moment kernel (F16) start
+// faster and have more in flight.  us, rows against the other: F32 aligned rows 64^3
+// 11.4 / 9.8, 72^3 12.4 / 12.6, 96^3 22.1 / 26.2; unaligned 70x71x72 15.7 / 11.7, 97^3
+// 31.3 / 27.3, 105^3 36.5 / 35.5, 113^3 43.9 / 48.3; F16 64^3 rows, 48^3 the moment
+// kernel.
+constexpr long long row_min_nodes(int prec, bool aligned) {
+  return prec == kF16 ? 190000 : aligned ? 350000 : 1200000;
 }
 
 struct RowPlan {
@@ -166,15 +174,14 @@ struct RowPlan {
 // fitted to 2300 measured cuts of 28 boxes, 24^3 to 256^3, odd and ragged ones among
 // them: the plan's choice is within 4% of the best cut of each, but for two FP16 boxes
 // (9%).
-inline RowPlan row_plan(int prec, int R, int nx, int ny, int nz, int sms) {
+inline RowPlan row_plan(int prec, int nx, int ny, int nz, int sms) {
+  constexpr int R = 1;   // E4 (E6 in rows: 256^3 730 us, the two passes 545)
   RowPlan best{false, false, 0, {0, 0, 0, 0}};
   const int es = prec == kF16 ? 2 : 4, ve = 16 / es;
   const bool aligned = nx % ve == 0;
   if (prec == kF64 || nx < 2 * R + 1 || ny < 2 * R + 1 || nz < 2 * R + 1) return best;
-  // smaller boxes stay with the moment kernel, whose CTAs start faster and are more
-  // (32^3 4.5 against 7.2 us, 48^3 7.8 against 8.4; 64^3 11.7 against 11.4)
-  if ((long long)nx * ny * nz < 190000) return best;
-  const RowCaps caps = row_caps(prec, R);
+  if ((long long)nx * ny * nz < row_min_nodes(prec, aligned)) return best;
+  const RowCaps caps = row_caps(prec);
   const double bytes = (double)nx * ny * nz * 38.0 * es;
   const double scale = (aligned ? 1.0 : 1.42) * (prec == kF16 ? 0.9 : 1.0);
   double best_t = 0.0;
@@ -214,6 +221,22 @@ inline long long lattice_grid_ctas(const LatticeDesc& d, TileCfg cfg) {
   return tiles * ((d.nz + cfg.zchunk - 1) / cfg.zchunk);
 }
 
+// Where the two-pass step (lbm_kernels_split.cuh) runs behind kinds 5 and 6, of the
+// boxes that the row kernel leaves: always in FP64; in FP32 with E6, and with E8 at
+// tau = 1; else up to 1.5 million nodes (the second pass's pull of the populations, or
+// the extra planes, miss L2 beyond.  us, two passes against the old kernel's best z
+// chunk, tau != 1: E4 64^3 12.0 / 14.8, 112^3 63.4 / 71.1, 120^3 77.9 / 73.3, 128^3
+// 92.9 / 86.9, 256^3 701 / 585; E8 112^3 89.8 / 105, 128^3 130 / 126, 192^3 423 / 383;
+// E6 128^3 95.6 / 114, 192^3 314 / 344).
+inline bool split_applies(int prec, int stencil, bool unit_tau, long long nodes) {
+  if (prec == kF64 || stencil == 6 || (stencil == 8 && unit_tau)) return true;
+  return nodes <= 1500000;
+}
+
+// The whole-row kernel (F32, F16; E4, tau = 1) where its plan has a cut of the box;
+// cudaErrorNotSupported (nothing launched) where it has not.
+cudaError_t launch_row_any(int prec, const LatticeDesc& d, bool prepare, cudaStream_t s);
+
 // ---------------------------------------------------------------- batches
 struct BatchEntry;
 struct BatchHeader;
@@ -233,7 +256,7 @@ constexpr bool batch_mode_row(int mode) { return mode == kBatchRow || mode == kB
 constexpr int kRowBatchDensityWarps = 9, kRowBatchCollideWarps = 6;
 inline int row_batch_rows(int prec, int stencil, int nx, int ny, int nz) {
   if (stencil != 4 || prec == kF64 || nx < 3 || ny < 3 || nz < 3) return 0;
-  const RowCaps caps = row_caps(prec, 1);
+  const RowCaps caps = row_caps(prec);
   const int ve = prec == kF16 ? 8 : 4;
   int most = (int)(((long long)kRowBatchDensityWarps * caps.kd * 64) / nx);
   if ((caps.slot - 4 * ve) / nx < most) most = (caps.slot - 4 * ve) / nx;
@@ -250,6 +273,8 @@ inline TileCfg batch_tile(int prec, int stencil, int mode) {
   t.kind = mode == kBatchMoment ? 5 : (mode == kBatchMomentElem ? 6 : 1);
   return t;
 }
+cudaError_t launch_row_batch_any(int prec, bool aligned, const BatchEntry* table, const BatchHeader* hdr, int step,
+                                 bool prepare, int* grid, cudaStream_t s);
 // items of one lattice in a batch launch of this mode, z chunks of zc planes; *rows as
 // for BatchEntry::rows
 inline long long batch_items(int prec, int stencil, int mode, int nx, int ny, int nz, int zc, int* rows) {

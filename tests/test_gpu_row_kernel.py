@@ -15,7 +15,18 @@ import paper_2105_08772_gb300 as P
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("box,prec,zc", [
+# boxes that take the two passes (lbm_kernels_split.cuh) where the others take the row
+# kernel, with their stencil and tau: for tau != 1 a fixed z chunk runs the chunked
+# (aligned rows) or the pipelined kernel
+OTHER = {
+    (72, 60, 64): ("E4", 0.8), (71, 60, 64): ("E4", 1.3), (3, 250, 261): ("E4", 0.7), (335, 41, 23): ("E4", 0.8),
+    (68, 60, 64): ("E6", 1.0), (69, 60, 64): ("E6", 1.0), (256, 31, 25): ("E6", 1.0), (8, 170, 150): ("E6", 1.0),
+    (3, 3, 3): ("E4", 1.0), (37, 29, 23): ("E4", 1.0), (100, 3, 4): ("E4", 1.0), (57, 57, 58): ("E4", 1.0),
+    (68, 64, 60): ("E8", 1.0), (61, 64, 60): ("E8", 1.0), (5, 201, 199): ("E8", 1.0), (68, 60, 63): ("E6", 0.8),
+}
+
+
+@pytest.mark.parametrize("box,prec,zc", [(b, "f32", min(8, b[2])) for b in OTHER] + [
     ((64, 56, 56), "f32", 8),        # aligned, 16 rows an item
     ((61, 60, 60), "f32", 8),        # unaligned rows
     ((127, 41, 43), "f32", 7),       # unaligned, ragged last row block and chunk
@@ -26,7 +37,18 @@ pytestmark = pytest.mark.gpu
     ((256, 256, 3), "f32", 3),       # three planes
     ((440, 24, 24), "f32", 8),       # long rows: two an item
     ((335, 41, 24), "f32", 8),
-    ((600, 20, 20), "f32", 8),       # too long: no cut, the moment kernel itself
+    ((600, 20, 20), "f32", 8),       # longer than a row item
+    ((76, 72, 70), "f32", 8),        # boxes from here on are large enough for rows in F32
+    ((107, 108, 109), "f32", 8),     # (above: the two passes)
+    ((127, 99, 97), "f32", 7),
+    ((4, 300, 300), "f32", 0),
+    ((3, 640, 641), "f32", 0),
+    ((200, 3, 600), "f32", 16),
+    ((201, 3, 2000), "f32", 16),
+    ((256, 456, 3), "f32", 3),
+    ((440, 30, 28), "f32", 8),
+    ((335, 41, 90), "f32", 8),
+    ((600, 51, 50), "f32", 8),       # too long, and too large for the two passes
     ((64, 64, 64), "f16", 8),
     ((56, 66, 60), "f16", 16),
     ((256, 40, 33), "f16", 16),
@@ -37,7 +59,8 @@ def test_row_kernel_is_bitwise_the_moment_kernel(box, prec, zc):
     rho = rho * (1.0 + 0.05 * rng.uniform(-1, 1, size=rho.shape))
     fields = []
     for fixed in (False, True):
-        lat = P.Lattice(*box, G=-5.0, prec=prec)
+        stencil, tau = OTHER.get(box, ("E4", 1.0))
+        lat = P.Lattice(*box, G=-5.0, prec=prec, stencil=stencil, tau=tau)
         try:
             code = lat.get_tile()
             assert code // 10 ** 8 in (5, 6) and code // 10 % 1000 == 0, code
