@@ -33,17 +33,18 @@ __device__ double density_at(const LatticeDesc& d, int x, int y, int z) {
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
     const int xx = wrap(x - cx(i), d.nx), yy = wrap(y - cy(i), d.ny), zz = wrap(z - cz(i), d.nz);
-    sum += (double)Storage<P>::load(src + (long long)i * d.plane + ((long long)zz * d.ny + yy) * d.nx + xx,
-                                    inv_scale);
+    sum += widen(Storage<P>::load(src + (long long)i * d.plane + ((long long)zz * d.ny + yy) * d.nx + xx, inv_scale));
   }
   return d.n0 + sum;
 }
 
+// One warp per sampled node, a lane per stencil vector: a node's 19 densities of 19
+// FP64 additions each would otherwise be one thread's chain (64 clocks an addition).
 template <int P, int ST>
 __global__ void point_obs_kernel(LatticeDesc d, PointOut* pts, double* n_line, double* PT_line,
                                  double* PN_line, int line_len) {
-  constexpr int R = stencil_radius<ST>();
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  constexpr int R = stencil_radius<ST>(), W1 = 2 * R + 1;
+  const int t = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (t >= 2 + line_len) return;
   const int c[3] = {d.nx / 2, d.ny / 2, d.nz / 2};
   int p[3];
@@ -56,20 +57,28 @@ __global__ void point_obs_kernel(LatticeDesc d, PointOut* pts, double* n_line, d
   } else {
     p[0] = (c[0] + (t - 2)) % d.nx; p[1] = c[1]; p[2] = c[2];
   }
-  const double n = density_at<P>(d, p[0], p[1], p[2]);
+  double n = 0.0, sxx = 0.0, syy = 0.0;
+  // vectors in raster order, those of the stencil dealt to the lanes in turn; the
+  // node itself goes to the last lane
+  if (lane == 31) n = density_at<P>(d, p[0], p[1], p[2]);
+  int mine = 0;
+  for (int k = 0; k < W1 * W1 * W1; ++k) {
+    const int dx = k % W1 - R, dy = k / W1 % W1 - R, dz = k / (W1 * W1) - R;
+    const double W = shell_weight<ST>(dx * dx + dy * dy + dz * dz);
+    if (W == 0.0) continue;
+    if (mine++ % 31 != lane) continue;
+    const double nb = density_at<P>(d, wrap(p[0] + dx, d.nx), wrap(p[1] + dy, d.ny), wrap(p[2] + dz, d.nz));
+    const double ps = W * psi_of<double>(nb, d.eos);
+    sxx += ps * (double)(dx * dx);
+    syy += ps * (double)(dy * dy);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    sxx += __shfl_xor_sync(0xffffffffu, sxx, o);
+    syy += __shfl_xor_sync(0xffffffffu, syy, o);
+  }
+  if (lane != 31) return;
   const double psic = psi_of<double>(n, d.eos);
-  double sxx = 0.0, syy = 0.0;
-  for (int dz = -R; dz <= R; ++dz)
-    for (int dy = -R; dy <= R; ++dy)
-      for (int dx = -R; dx <= R; ++dx) {
-        const double W = shell_weight<ST>(dx * dx + dy * dy + dz * dz);
-        if (W == 0.0 || (dx == 0 && dy == 0 && dz == 0)) continue;
-        const double nb = density_at<P>(d, wrap(p[0] + dx, d.nx), wrap(p[1] + dy, d.ny),
-                                        wrap(p[2] + dz, d.nz));
-        const double ps = psi_of<double>(nb, d.eos);
-        sxx += W * ps * (double)(dx * dx);
-        syy += W * ps * (double)(dy * dy);
-      }
   const double k = 0.5 * d.eos.G * (1.0 / 3.0) * psic;
   const double Pxx = n * (1.0 / 3.0) + k * sxx;
   const double Pyy = n * (1.0 / 3.0) + k * syy;
@@ -97,35 +106,52 @@ __global__ void finalize_kernel(FinalizeArgs a) {
     }
     __syncthreads();
   }
+  // trapezoid rule on r = 0..line_len-1, and the closed forms in warps of their own:
+  // one thread's FP64 chain is what this kernel's time is
+  const PointOut pt = *a.pts;
+  __shared__ double line[2][NT], form[8];
+  {
+    double C = 0.0, D = 0.0;
+    for (int r = t; r < a.line_len; r += NT) {
+      const double g = pt.P_out - a.PT_line[r];
+      const double wt = (r == 0 || r == a.line_len - 1) ? 0.5 : 1.0;
+      C += wt * (double)r * (double)r * g;
+      D += wt * (double)r * g;
+    }
+    line[0][t] = C;
+    line[1][t] = D;
+  }
+  __syncthreads();
+  for (int off = NT / 2; off > 0; off >>= 1) {
+    if (t < off) {
+      line[0][t] += line[0][t + off];
+      line[1][t] += line[1][t + off];
+    }
+    __syncthreads();
+  }
+  const double V = (double)a.volume, dP = pt.P_in - pt.P_out;
+  const double q = (dP != 0.0) ? line[0][0] / dP : -1.0;
+  // centre of mass of n - n_out: mean minimum-image displacement
+  if (t == 0 || t == 32 || t == 64) form[t / 32] = red[2 + t / 32][0] / red[1][0];
+  if (t == 96) form[3] = cbrt(3.0 * (red[0][0] - V * pt.n_out) / (4.0 * M_PI * (pt.n_in - pt.n_out)));
+  if (t == 128) form[4] = q > 0.0 ? cbrt(6.0 * q) : NAN;
+  __syncthreads();
   if (t != 0) return;
   lbm_obs o;
-  const PointOut pt = *a.pts;
   o.n_in = pt.n_in;
   o.n_out = pt.n_out;
   o.P_in = pt.P_in;
   o.P_out = pt.P_out;
-  o.dP = pt.P_in - pt.P_out;
+  o.dP = dP;
   o.mass = red[0][0];
-  const double wsum = red[1][0];
-  // centre of mass of n - n_out: centre node + mean minimum-image displacement
-  double rel[3] = {red[2][0] / wsum, red[3][0] / wsum, red[4][0] / wsum};
+  const double rel[3] = {form[0], form[1], form[2]};
   for (int k = 0; k < 3; ++k) o.com[k] = (double)a.center[k] + rel[k];
-  const double V = (double)a.volume;
-  o.R_e = cbrt(3.0 * (o.mass - V * o.n_out) / (4.0 * M_PI * (o.n_in - o.n_out)));
-  // trapezoid rule on r = 0..line_len-1
-  double C = 0.0, D = 0.0;
-  for (int r = 0; r < a.line_len; ++r) {
-    const double g = o.P_out - a.PT_line[r];
-    const double wt = (r == 0 || r == a.line_len - 1) ? 0.5 : 1.0;
-    C += wt * (double)r * (double)r * g;
-    D += wt * (double)r * g;
-  }
-  o.C = C;
-  o.D = D;
-  const double q = (o.dP != 0.0) ? C / o.dP : -1.0;
+  o.R_e = form[3];
+  o.C = line[0][0];
+  o.D = line[1][0];
   unsigned st = 0;
   if (q > 0.0) {
-    o.R_s = cbrt(6.0 * q);
+    o.R_s = form[4];
     o.sigma_s = 0.5 * o.dP * o.R_s;
   } else {
     o.R_s = NAN;
@@ -154,7 +180,7 @@ cudaError_t launch_point_obs(int prec, int stencil, const LatticeDesc& d, PointO
                              double* n_line, double* PT_line, double* PN_line, cudaStream_t s) {
   const int line_len = d.nx / 2 + 1;
   const int n = 2 + line_len;
-  const dim3 grid((n + 63) / 64);
+  const dim3 grid((n + 1) / 2);   // two warps a block
 #define LBM_POINT(PR, STC) \
   point_obs_kernel<PR, STC><<<grid, 64, 0, s>>>(d, pts, n_line, PT_line, PN_line, line_len)
   if (stencil != 4 && stencil != 6 && stencil != 8) return cudaErrorInvalidValue;
