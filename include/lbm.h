@@ -117,8 +117,10 @@ typedef struct {
 /* ---------------------------------------------------------------- set-up */
 
 /* Bytes of device workspace one lattice needs (two population buffers of
- * 19 planes, a velocity snapshot for delta u, reduction scratch, for F64 and
- * F32 a plane of psi).  Returns 0 for invalid arguments. */
+ * 19 planes, a velocity snapshot for delta u, reduction scratch, for F64 and most
+ * F32 boxes a plane of psi).  lbm_create also takes a workspace without that last
+ * plane (nodes * storage bytes, rounded up to 256): steps then run the kernels that
+ * need none.  Returns 0 for invalid arguments. */
 size_t lbm_workspace_bytes(lbm_box box, int stencil, int prec);
 
 /* Create a context for one periodic lattice (Sec. II).  tau: BGK relaxation

@@ -124,7 +124,9 @@ struct Layout {
   long long npart;
 };
 
-Layout layout_of(lbm_box b, int prec) {
+// aux, the last region, is optional: without it the kernels that need no psi plane run.
+// FP32 boxes that never take the two passes have none (split_applies).
+Layout layout_of(lbm_box b, int stencil, int prec) {
   Layout L;
   const size_t N = (size_t)b.nx * b.ny * b.nz;
   L.npart = obs_partials(b, default_obs_zchunk(b));
@@ -134,7 +136,7 @@ Layout layout_of(lbm_box b, int prec) {
   // state block: PointOut at 0, dP_prev at kStateDP, the lbm_obs record at kStateObs
   L.state = align256(kStateObs + sizeof(lbm_obs));
   L.lines = align256(3 * sizeof(double) * (size_t)(b.nx / 2 + 1));
-  L.aux = prec == kF16 ? 0 : align256(N * storage_bytes(prec));
+  L.aux = prec == kF16 || !split_applies(prec, stencil, stencil != 4, (long long)N) ? 0 : align256(N * storage_bytes(prec));
   L.total = 2 * L.pop + L.u_old + L.partials + L.state + L.lines + L.aux;
   return L;
 }
@@ -509,7 +511,7 @@ extern "C" {
 
 size_t lbm_workspace_bytes(lbm_box box, int stencil, int prec) {
   if (!valid_stencil(stencil) || !valid_prec(prec) || !box_ok(box, stencil)) return 0;
-  return layout_of(box, prec).total;
+  return layout_of(box, stencil, prec).total;
 }
 
 lbm_status lbm_create(lbm_box box, double tau, double G, lbm_eos eos, int stencil, int prec,
@@ -537,11 +539,11 @@ lbm_status lbm_create(lbm_box box, double tau, double G, lbm_eos eos, int stenci
   } else {
     return fail(nullptr, LBM_EINVAL, "unknown psi kind %d", eos.kind);
   }
-  const Layout L = layout_of(box, prec);
+  const Layout L = layout_of(box, stencil, prec);
   if (!dev_workspace) return fail(nullptr, LBM_EINVAL, "workspace is null");
   if (((uintptr_t)dev_workspace & 255) != 0) return fail(nullptr, LBM_EINVAL, "workspace not 256-byte aligned");
-  if (bytes < L.total)
-    return fail(nullptr, LBM_ENOMEM, "workspace has %zu bytes, needs %zu", bytes, L.total);
+  if (bytes < L.total - L.aux)
+    return fail(nullptr, LBM_ENOMEM, "workspace has %zu bytes, needs %zu", bytes, L.total - L.aux);
 
   lbm_ctx* c = new lbm_ctx();
   memset(c->err, 0, sizeof(c->err));
@@ -570,7 +572,7 @@ lbm_status lbm_create(lbm_box box, double tau, double G, lbm_eos eos, int stenci
   c->PT_line = c->n_line + c->line_len;
   c->PN_line = c->PT_line + c->line_len;
   p += L.lines;
-  c->aux = L.aux ? p : nullptr;
+  c->aux = L.aux && bytes >= L.total ? p : nullptr;
   c->cur = 0;
   c->n0 = 0.0;
   c->scale = 1.0;
@@ -1438,7 +1440,8 @@ struct BatchLayout {
 
 BatchLayout batch_layout(int slots, lbm_box max_box, int stencil, int prec) {
   BatchLayout L;
-  L.slot = lbm_workspace_bytes(max_box, stencil, prec);
+  const Layout one = layout_of(max_box, stencil, prec);
+  L.slot = one.total - one.aux;   // the batch kernels need no psi plane
   L.table = align256(sizeof(BatchEntry) * (size_t)slots);
   L.hdr = align256(sizeof(BatchHeader));
   L.total = L.slot * (size_t)slots + L.table + L.hdr;

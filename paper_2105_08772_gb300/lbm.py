@@ -454,7 +454,16 @@ class Lattice:
         self.nbytes = lbm_workspace_bytes(self.box, st, pr)
         if self.nbytes == 0:
             raise LBMError(_lib.LBM_EINVAL, "invalid box/stencil/precision")
-        self.workspace = torch.empty(self.nbytes + 256, dtype=torch.uint8, device="cuda")
+        try:
+            self.workspace = torch.empty(self.nbytes + 256, dtype=torch.uint8, device="cuda")
+        except torch.cuda.OutOfMemoryError:
+            # a box that only just fits: lbm_create does without the psi plane at the end
+            # (F64, F32 with a wide stencil; large E4 boxes have none)
+            if self.prec == "f16" or (self.prec, self.stencil) == ("f32", "E4"):
+                raise
+            plane = self.nx * self.ny * self.nz * (8 if self.prec == "f64" else 4)
+            self.nbytes -= plane + (-plane) % 256
+            self.workspace = torch.empty(self.nbytes + 256, dtype=torch.uint8, device="cuda")
         ptr = self.workspace.data_ptr()
         ptr += (-ptr) % 256
         s = self.stream if self.stream is not None else torch.cuda.current_stream()
