@@ -57,10 +57,13 @@ def measured_peak_gbs():
 
 
 KERNEL_SOURCES = ("lbm_common.cuh", "lbm_exptab.cuh", "lbm_math.cuh", "lbm_kernels.cuh", "lbm_kernels_async.cuh", "lbm_kernels_chunk.cuh",
-                  "lbm_kernels_moment.cuh", "lbm_kernels_tma.cuh", "lbm_kernels_row.cuh", "lbm_kernels_split.cuh", "lbm_launch.h", "lbm_lattice_inst.cuh")
+                  "lbm_kernels_moment.cuh", "lbm_kernels_tma.cuh", "lbm_kernels_row.cuh", "lbm_kernels_split.cuh",
+                  "lbm_row.cu", "lbm_step_launch.h", "lbm_launch.h", "lbm_lattice_inst.cuh")
 
 
-PROFILE_STEMS = {7: "lattice_tma", 6: "lattice_moment_elem", 5: "lattice_moment"}
+# the row kernel's summary first: it is what kinds 5 and 6 run on the FP32 and FP16
+# workloads without a fixed z chunk
+PROFILE_STEMS = {7: ("lattice_tma",), 6: ("lattice_row", "lattice_moment_elem"), 5: ("lattice_row", "lattice_moment")}
 
 
 def profile_fields(stem, prec, box=128):
@@ -88,8 +91,8 @@ def measured_traffic(prec, kind=5):
     """DRAM bytes per launch of the step kernel from the committed ncu summary of the
     128^3 workload, or None when there is none for this kernel and precision or the
     kernel sources changed since."""
-    stem = PROFILE_STEMS.get(int(kind))
-    fields = profile_fields(stem, prec) if stem else None
+    found = (profile_fields(stem, prec) for stem in PROFILE_STEMS.get(int(kind), ()))
+    fields = next((f for f in found if f), None)
     if not fields or "traffic_bytes_per_launch" not in fields:
         return None
     return int(fields["traffic_bytes_per_launch"])
@@ -100,7 +103,7 @@ def fp64_bound(hbm_gbs, peak):
     from the committed ncu summary when it was taken on the current sources (else
     the bound is left null)."""
     frac = hbm_gbs / peak
-    prof = profile_fields("lattice_moment", "f64")
+    prof = profile_fields("split", "f64") or profile_fields("lattice_moment", "f64")
     pipe = float(prof["fp64_pipe_pct"]) if prof and "fp64_pipe_pct" in prof else None
     bound = None
     evidence = f"this run: DRAM at {100 * frac:.1f}% of the measured HBM peak"
@@ -112,8 +115,8 @@ def fp64_bound(hbm_gbs, peak):
 
 KERNEL_KINDS = {
     7: "lattice_tma_kernel (TMA tensor-tile pull + on-chip psi halo + SC force + Guo-BGK at tau = 1 + store)",
-    6: "lattice_moment_kernel, element copies (pull + on-chip psi halo + SC force + Guo-BGK at tau = 1 + store)",
-    5: "lattice_moment_kernel, row chunks (pull + on-chip psi halo + SC force + Guo-BGK at tau = 1 + store)",
+    6: "lattice_row_kernel (FP64: split kernels), else lattice_moment_kernel with element copies (pull + on-chip psi halo + SC force + Guo-BGK at tau = 1 + store)",
+    5: "lattice_row_kernel (FP64: split kernels), else lattice_moment_kernel with row chunks (pull + on-chip psi halo + SC force + Guo-BGK at tau = 1 + store)",
     4: "lattice_chunk_kernel", 1: "lattice_async_kernel", 0: "lattice_kernel",
 }
 
