@@ -66,6 +66,7 @@ struct EosParams {
   // the same constants rounded to float on the host (set_float_params), so that
   // FP32 kernels take them straight from the parameter bank and convert nothing
   float Gf, af, bf, RTf;
+  float Glo;      // what Gf lost of G
 };
 
 template <typename T>
@@ -151,10 +152,20 @@ inline void set_float_params(LatticeDesc& d) {
   d.scalef = (float)d.scale;
   d.inv_scalef = (float)(1.0 / d.scale);
   d.eos.Gf = (float)d.eos.G;
+  d.eos.Glo = (float)(d.eos.G - (double)d.eos.Gf);
   d.eos.af = (float)d.eos.a;
   d.eos.bf = (float)d.eos.b;
   d.eos.RTf = (float)(d.eos.Rgas * d.eos.T);
 }
+
+// G in the kernel's arithmetic type, and what that rounding lost of it.
+template <typename T> struct Coupling {
+  T G, lo;
+  __device__ __forceinline__ explicit Coupling(const EosParams& e) {
+    if constexpr (sizeof(T) == 8) { G = e.G; lo = 0; }
+    else { G = e.Gf; lo = e.Glo; }
+  }
+};
 
 // A descriptor parameter in the kernel's arithmetic type: the host-rounded float
 // copy for FP32 arithmetic, the double itself for FP64.

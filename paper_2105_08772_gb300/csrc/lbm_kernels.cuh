@@ -106,7 +106,7 @@ __device__ __forceinline__ void load_plane(const LatticeDesc& d, int x0, int y0,
 // formed those values and kept them in registers); differences along the node's
 // own column take them from there instead of from shared memory.
 template <typename T, int ST, int PX, bool OWN = false>
-__device__ __forceinline__ void sc_force_pairs(const T* const* planes, T G, T& Fx, T& Fy, T& Fz,
+__device__ __forceinline__ void sc_force_pairs(const T* const* planes, Coupling<T> G, T& Fx, T& Fy, T& Fz,
                                                const T* own = nullptr) {
   constexpr int R = stencil_radius<ST>();
   auto at = [&](int dx, int dy, int dz) {
@@ -120,7 +120,7 @@ __device__ __forceinline__ void sc_force_pairs(const T* const* planes, T G, T& F
 // slots[k] is the ring slot of plane z + k - R.
 template <int P, int ST, int BX, int BY>
 __device__ __forceinline__ void sc_force(const typename Storage<P>::T* ring, const int* slots, int tx,
-                                         int ty, typename Storage<P>::T G,
+                                         int ty, Coupling<typename Storage<P>::T> G,
                                          typename Storage<P>::T& Fx, typename Storage<P>::T& Fy,
                                          typename Storage<P>::T& Fz) {
   using Sh = StepShape<P, ST, BX, BY>;
@@ -200,7 +200,8 @@ lattice_kernel(LatticeDesc d, int zchunk, ObsArgs oa) {
                               pops + ((kk + NP) % NP) * Q * NT, kk >= 0 && kk < zc);
   }
 
-  const T G = dparam<T>(d.eos.G, d.eos.Gf), omega = dparam<T>(d.omega, d.omegaf), n0 = dparam<T>(d.n0, d.n0f);
+  const Coupling<T> G(d.eos);
+  const T omega = dparam<T>(d.omega, d.omegaf), n0 = dparam<T>(d.n0, d.n0f);
   const T scale = dparam<T>(d.scale, d.scalef);
   const long long plane = d.plane;
   double acc_mass = 0, acc_w = 0, acc_wz = 0, acc_du = 0, acc_max = 0;   // acc_max: |u|^2

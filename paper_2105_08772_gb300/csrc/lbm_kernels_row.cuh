@@ -36,7 +36,7 @@
 // step, 1.00 of the measured copy rate; 192^3 171 us, 0.92; the moment kernel 481 and
 // 214); an SM's own time per plane (loads and stores of shared memory, latency) for
 // FP16 (192^3 96.5 us, 0.82; 154.9) and unaligned rows (157^3 100 us, 0.87; 142);
-// the step's latency below 100^3 (64^3 11.4 us; 14.1).
+// the step's latency below 100^3 (96^3 22.1 us; 30.3).
 // What did not help: four x-neighbours a thread with 16-byte accesses (128^3 67 us
 // against 54: bank conflicts of their outer neighbours, half the warps), two CTAs of
 // half the size per SM, a second stage, stores through bulk copies (18 B/clk).
@@ -438,7 +438,8 @@ __device__ __forceinline__ void row_process_item(const LatticeDesc& d, const Row
   }
 
   // collision warps
-  const T G = dparam<T>(d.eos.G, d.eos.Gf), scale = dparam<T>(d.scale, d.scalef);
+  const Coupling<T> G(d.eos);
+  const T scale = dparam<T>(d.scale, d.scalef);
   const int tc = tid - c.nd;
   const int inner = h * nx;
   const long long pbytes = d.plane * (long long)sizeof(S);

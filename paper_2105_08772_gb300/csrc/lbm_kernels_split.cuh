@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(128) split_collide_kernel(LatticeDesc d) {
   const T* psi = static_cast<const T*>(d.aux);
   auto at = [&](int dx, int dy, int dz) { return __ldg(psi + (zo[dz + R] + yo[dy + R] + xo[dx + R])); };
   T Fx, Fy, Fz;
-  sc_force_at<T, ST>(at, at(0, 0, 0), dparam<T>(d.eos.G, d.eos.Gf), Fx, Fy, Fz);
+  sc_force_at<T, ST>(at, at(0, 0, 0), Coupling<T>(d.eos), Fx, Fy, Fz);
   collide_nodes<T, UNIT, false>(
       dn, vadd(dparam<T>(d.n0, d.n0f), dn), jx, jy, jz, Fx, Fy, Fz, dparam<T>(d.omega, d.omegaf), (T)1,
       [&](int i) { return old[UNIT ? 0 : i]; }, [&](int i, T g) { out[i * d.plane] = g; });

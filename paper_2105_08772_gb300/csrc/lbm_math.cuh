@@ -166,9 +166,18 @@ __device__ __forceinline__ V sc_force_axis(At at, int axis) {
 }
 
 template <typename V, int ST, typename At>
-__device__ __forceinline__ void sc_force_at(At at, V psi0, typename Lane<V>::T G, V& Fx, V& Fy, V& Fz) {
+__device__ __forceinline__ void sc_force_at(At at, V psi0, Coupling<typename Lane<V>::T> cpl, V& Fx, V& Fy, V& Fz) {
   using T = typename Lane<V>::T;
-  const V k = vmul(Lane<V>::all(-G * (T)(1.0 / (3.0 * shell_denominator<ST>()))), psi0);
+  constexpr double c = 1.0 / (3.0 * shell_denominator<ST>());
+  const T hi = -cpl.G * (T)c;
+  V k = vmul(Lane<V>::all(hi), psi0);
+  if constexpr (sizeof(T) == 4) {
+    // FP32: what the rounding of G and of the constant lost.  Left out it is a G off by
+    // up to 1e-7 at every node and step, which the interface amplifies (48x40x44 bubble,
+    // 160 steps: populations off by 5e-5).
+    const T lo = vfma(-cpl.G, (T)c, -hi) - vfma(cpl.G, (T)(c - (double)(T)c), cpl.lo * (T)c);
+    k = vfma(Lane<V>::all(lo), psi0, k);
+  }
   Fx = vmul(k, sc_force_axis<V, ST>(at, 0));
   Fy = vmul(k, sc_force_axis<V, ST>(at, 1));
   Fz = vmul(k, sc_force_axis<V, ST>(at, 2));
@@ -185,8 +194,9 @@ __device__ __forceinline__ void sc_force_at(At at, V psi0, typename Lane<V>::T G
 //   omega g_i^eq + F_i = w_i [base + 9/2 (e.u)(e.q) + 3 e.p],
 // which takes half the operations of forming g_i^eq and F_i one by one (the FP64
 // step is bound by its FP64 instructions and the FP16 step by instruction issue).
-// Scaled to the diagonal weight 1/36: B = base/36, U = u/8, P = p/12; an axis
-// population is twice [B + U_a q_a +- P_a].  Opposite velocities share the even
+// Scaled to the diagonal weight 1/36: B = base/36, U = u/8, P = p/36; an axis
+// population is twice [B + U_a q_a +- 3 P_a].  (P = p/12 would scale every momentum by
+// the error of 1/12 in FP32, 3.0e-8, four times that of 1/36.)  Opposite velocities share the even
 // part; the odd part flips sign.
 //
 // Mass closure: sum g*_i = dn holds exactly for exact weights, but the rounded
@@ -227,11 +237,11 @@ __device__ __forceinline__ void collide_nodes(V dn, V n, V jx, V jy, V jz, V Fx,
   const V uq = vfma(uz, qz, vfma(uy, qy, vmul(ux, qx)));
   base = vfma(L::all((T)-1.5), uq, base);
   const T s = SCALED ? wscale : (T)1;
-  const V B = vmul(base, L::all((T)(1.0 / 36.0) * s));
-  const V c8 = L::all((T)0.125 * s), c12 = L::all((T)(1.0 / 12.0) * s);
+  const V c8 = L::all((T)0.125 * s), c36 = L::all((T)(1.0 / 36.0) * s);
+  const V B = vmul(base, c36);
   const V Ux = vmul(ux, c8), Uy = vmul(uy, c8), Uz = vmul(uz, c8);
-  px = vmul(px, c12); py = vmul(py, c12); pz = vmul(pz, c12);
-  const V two = L::all((T)2), vom1 = L::all(om1);
+  px = vmul(px, c36); py = vmul(py, c36); pz = vmul(pz, c36);
+  const V two = L::all((T)2), three = L::all((T)3), six = L::all((T)6), vom1 = L::all(om1);
   // One opposite pair: g*_i, g*_{i+1} and its even part ev (an axis pair: twice the
   // diagonal one, formed with one fused operation each).  Without omega = 1 the old
   // populations' share is added, and the pair's sum (2 ev, or 4 ev for an axis) takes
@@ -249,12 +259,12 @@ __device__ __forceinline__ void collide_nodes(V dn, V n, V jx, V jy, V jz, V Fx,
     }
   };
   auto axis = [&](int i, V U, V q, V P) {
-    const V ev = vfma(U, q, B), P2 = vadd(P, P);
+    const V ev = vfma(U, q, B), P2 = vmul(six, P);
     return pair(i, vfma(two, ev, P2), vsub(vadd(ev, ev), P2), ev, (T)4);
   };
   auto diag = [&](int i, V U, V q, V P) {
     const V ev = vfma(U, q, B);
-    return pair(i, vadd(ev, P), vsub(ev, P), ev, (T)2);
+    return pair(i, vfma(three, P, ev), vfma(L::all((T)-3), P, ev), ev, (T)2);
   };
   const V a12 = axis(1, Ux, qx, px), a34 = axis(3, Uy, qy, py), a56 = axis(5, Uz, qz, pz);
   const V d78 = diag(7, vadd(Ux, Uy), vadd(qx, qy), vadd(px, py));
