@@ -66,7 +66,7 @@ struct EosParams {
   // the same constants rounded to float on the host (set_float_params), so that
   // FP32 kernels take them straight from the parameter bank and convert nothing
   float Gf, af, bf, RTf;
-  float Glo;      // what Gf lost of G
+  float Khi[3], Klo[3];   // -G / (3 denominator) of E4, E6, E8 as the sum of two floats
 };
 
 template <typename T>
@@ -152,19 +152,22 @@ inline void set_float_params(LatticeDesc& d) {
   d.scalef = (float)d.scale;
   d.inv_scalef = (float)(1.0 / d.scale);
   d.eos.Gf = (float)d.eos.G;
-  d.eos.Glo = (float)(d.eos.G - (double)d.eos.Gf);
+  const double den[3] = {12.0, 120.0, 5040.0};   // shell_denominator
+  for (int k = 0; k < 3; ++k) {
+    const double K = -d.eos.G / (3.0 * den[k]);
+    d.eos.Khi[k] = (float)K;
+    d.eos.Klo[k] = (float)(K - (double)d.eos.Khi[k]);
+  }
   d.eos.af = (float)d.eos.a;
   d.eos.bf = (float)d.eos.b;
   d.eos.RTf = (float)(d.eos.Rgas * d.eos.T);
 }
 
-// G in the kernel's arithmetic type, and what that rounding lost of it.
+// The force's constant of a stencil: FP32 reads the host's two floats from the
+// parameter bank (no registers), FP64 forms it from G.
 template <typename T> struct Coupling {
-  T G, lo;
-  __device__ __forceinline__ explicit Coupling(const EosParams& e) {
-    if constexpr (sizeof(T) == 8) { G = e.G; lo = 0; }
-    else { G = e.Gf; lo = e.Glo; }
-  }
+  const EosParams& e;
+  __device__ __forceinline__ explicit Coupling(const EosParams& eos) : e(eos) {}
 };
 
 // A descriptor parameter in the kernel's arithmetic type: the host-rounded float

@@ -168,15 +168,15 @@ __device__ __forceinline__ V sc_force_axis(At at, int axis) {
 template <typename V, int ST, typename At>
 __device__ __forceinline__ void sc_force_at(At at, V psi0, Coupling<typename Lane<V>::T> cpl, V& Fx, V& Fy, V& Fz) {
   using T = typename Lane<V>::T;
-  constexpr double c = 1.0 / (3.0 * shell_denominator<ST>());
-  const T hi = -cpl.G * (T)c;
-  V k = vmul(Lane<V>::all(hi), psi0);
+  V k;
   if constexpr (sizeof(T) == 4) {
-    // FP32: what the rounding of G and of the constant lost.  Left out it is a G off by
-    // up to 1e-7 at every node and step, which the interface amplifies (48x40x44 bubble,
-    // G -4.6, 160 steps: populations off by 2.3e-5, now 2.9e-6).
-    const T lo = vfma(-cpl.G, (T)c, -hi) - vfma(cpl.G, (T)(c - (double)(T)c), cpl.lo * (T)c);
-    k = vfma(Lane<V>::all(hi), psi0, vmul(Lane<V>::all(lo), psi0));   // lo psi0 is below k's last place: one rounding
+    // FP32: in two floats, one rounding.  One float is a G off by up to 1e-7 at every node
+    // and step, which the interface amplifies (48x40x44 bubble, G -4.6, 160 steps:
+    // populations off by 2.3e-5, now 2.9e-6).
+    constexpr int i = ST == 4 ? 0 : (ST == 6 ? 1 : 2);
+    k = vfma(Lane<V>::all(cpl.e.Khi[i]), psi0, vmul(Lane<V>::all(cpl.e.Klo[i]), psi0));
+  } else {
+    k = vmul(Lane<V>::all(-cpl.e.G * (T)(1.0 / (3.0 * shell_denominator<ST>()))), psi0);
   }
   Fx = vmul(k, sc_force_axis<V, ST>(at, 0));
   Fy = vmul(k, sc_force_axis<V, ST>(at, 1));
