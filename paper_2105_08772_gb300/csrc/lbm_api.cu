@@ -1993,16 +1993,19 @@ lbm_status lbm_group_step(lbm_group* g, long long n) {
   for (lbm_ctx* c : g->ctx)
     if (!c->initialised) return gfail(g, LBM_EINVAL, "a lattice of the group is not initialised");
   if (n == 0) return LBM_OK;
-  // the table holds each lattice's buffer parity: write it again (and drop the
-  // graph captured with the old table) when any lattice's parity has changed, e.g.
-  // after an odd number of steps or a lattice stepped on its own
+  // the table holds each lattice's buffer parity and storage shift and scale: write it
+  // again when any of them has changed, e.g. after an odd number of steps, a lattice
+  // stepped on its own, initialised again or loaded.  (A captured graph holds the
+  // table's address only and stays valid.)
   bool stale = g->table_host.size() != g->ctx.size();
-  for (size_t k = 0; !stale && k < g->ctx.size(); ++k) stale = g->table_host[k].parity != g->ctx[k]->cur;
+  for (size_t k = 0; !stale && k < g->ctx.size(); ++k) {
+    const BatchEntry& e = g->table_host[k];
+    const lbm_ctx* c = g->ctx[k];
+    stale = e.parity != c->cur || e.d.n0 != c->n0 || e.d.scale != c->scale;
+  }
   if (stale) {
     lbm_status st = group_upload(g);
     if (st != LBM_OK) return st;
-    if (g->graph) cudaGraphExecDestroy(g->graph);
-    g->graph = nullptr;
   }
   if (n >= g->graph_len && !g->graph) {
     cudaGraph_t gr = nullptr;
