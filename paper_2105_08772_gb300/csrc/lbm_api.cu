@@ -1448,54 +1448,17 @@ BatchLayout batch_layout(int slots, lbm_box max_box, int stencil, int prec) {
   return L;
 }
 
-// kernel mode of the whole queue: the moment kernel needs tau = 1 and boxes whose
-// rows split into 16-byte chunks (nx % 4 == 0) at least a tile plus apron wide
-int natural_batch_mode(const lbm_batch* b);
-
-// the kernel modes that can run the whole queue, fastest first by construction
-std::vector<int> batch_modes_allowed(int natural, int prec) {
-  if (prec == kF16) return natural == kBatchRow ? std::vector<int>{kBatchRow, kBatchMoment}
-                                                : std::vector<int>{kBatchMoment};
-  if (natural == kBatchRow) return {kBatchRow, kBatchMoment, kBatchUnitTau};
-  if (natural == kBatchRowAny) return {kBatchRowAny, kBatchMomentElem, kBatchUnitTau};
-  if (natural == kBatchMoment) return {kBatchMoment, kBatchMomentElem, kBatchUnitTau};
-  if (natural == kBatchMomentElem) return {kBatchMomentElem, kBatchUnitTau};
-  return {natural};
-}
-
-int batch_mode(const lbm_batch* b) {
-  const int natural = natural_batch_mode(b);
-  if (b->mode_override >= 0)
-    for (int m : batch_modes_allowed(natural, b->prec))
-      if (m == b->mode_override) return m;
-  return natural;
-}
-
-// The mode of a set of lattices: the row kernel where it takes every box and the
-// lattices together are worth its few large items (a launch of 152 CTAs; below
-// 190000 nodes in all the tile kernels' many small CTAs are faster).
-struct BatchMix {
-  int prec, stencil;
-  bool unit = true, moment = true, aligned = true, rows = true;
-  double nodes = 0.0;
-  void add(lbm_box box, double tau) {
-    const int bx = batch_tile(prec, stencil, kBatchMoment).bx;
-    if (tau != 1.0) unit = false;
-    if (box.nx % 4 != 0 || box.nx < bx + 8) moment = false;
-    if (box.nx % (prec == kF16 ? 8 : 4) != 0) aligned = false;
-    if (row_batch_rows(prec, stencil, box.nx, box.ny, box.nz) == 0) rows = false;
-    nodes += (double)box.nx * box.ny * box.nz;
-  }
-  int mode() const {
-    if (!unit) return kBatchMixedTau;
-    if (rows && nodes >= 190000.0) return aligned ? kBatchRow : kBatchRowAny;
-    return moment ? kBatchMoment : kBatchMomentElem;
-  }
-};
-
-int natural_batch_mode(const lbm_batch* b) {
+// the whole queue as a mix of lattices
+BatchMix queue_mix(const lbm_batch* b) {
   BatchMix m{b->prec, b->stencil};
-  for (const BatchRun& r : b->runs) m.add(r.box, r.tau);
+  for (const BatchRun& r : b->runs) m.add(r.box.nx, r.box.ny, r.box.nz, r.tau);
+  return m;
+}
+
+// the kernel mode of the queue: the tuned one while every run of the queue allows it
+int batch_mode(const lbm_batch* b) {
+  const BatchMix m = queue_mix(b);
+  if (b->mode_override >= 0 && m.takes(b->mode_override)) return b->mode_override;
   return m.mode();
 }
 
@@ -1568,6 +1531,8 @@ lbm_status batch_upload(lbm_batch* b) {
   for (int k = 0; k < b->slots; ++k) {
     lbm_ctx* c = b->slot_ctx[k];
     if (!c) continue;
+    if (!batch_mode_takes(b->prec, b->stencil, b->graph_mode, c->box.nx, c->box.ny, c->box.nz, c->tau))
+      return bfail(b, LBM_EINVAL, "the batch's kernel does not take the box %dx%dx%d", c->box.nx, c->box.ny, c->box.nz);
     BatchEntry e;
     e.d = desc_of(c, 0);
     e.parity = c->cur;
@@ -1770,7 +1735,8 @@ lbm_status lbm_batch_autotune(lbm_batch* b, int reps, long long* choice) {
   for (int k = 0; k < b->slots; ++k)
     if (b->slot_ctx[k]) filled.push_back(k);
   if (filled.empty()) return bfail(b, LBM_EINVAL, "autotune needs queued runs");
-  const int natural = natural_batch_mode(b);
+  const BatchMix mix = queue_mix(b);
+  const int natural = mix.mode();
   std::vector<int> caps = {b->slots};
   if ((int)filled.size() >= 4) caps.push_back((b->slots + 1) / 2);
   cudaEvent_t e0, e1;
@@ -1779,7 +1745,8 @@ lbm_status lbm_batch_autotune(lbm_batch* b, int reps, long long* choice) {
   int best_mode = natural, best_zc = 0, best_cap = b->slots;
   double best_rate = -1.0;
   const int save_cap = b->slot_cap;
-  for (int mode : batch_modes_allowed(natural, b->prec)) {
+  for (int mode = kBatchModes - 1; mode >= 0; --mode) {
+    if (!mix.candidate(mode)) continue;
     for (int zc : {8, 16, 32}) {
       for (int cap : caps) {
         b->mode_override = mode;
@@ -1965,7 +1932,7 @@ lbm_status lbm_group_create(lbm_ctx* const* ctxs, int n, void* dev_workspace, si
   g->table_dev = reinterpret_cast<BatchEntry*>(ws);
   g->hdr_dev = reinterpret_cast<BatchHeader*>(ws + align256(sizeof(BatchEntry) * (size_t)n));
   BatchMix mix{g->prec, g->stencil};   // kernel mode as for a batch
-  for (lbm_ctx* c : g->ctx) mix.add(c->box, c->tau);
+  for (lbm_ctx* c : g->ctx) mix.add(c->box.nx, c->box.ny, c->box.nz, c->tau);
   g->mode = mix.mode();
   cudaError_t e = cudaStreamCreateWithFlags(&g->cap_stream, cudaStreamNonBlocking);
   if (e == cudaSuccess)

@@ -242,13 +242,12 @@ struct BatchEntry;
 struct BatchHeader;
 // the tile every batch of this precision / stencil uses, and its launch;
 // prepare readies the kernel outside capture and reports the grid it uses
-// batch kernel modes: lattices with mixed tau, all tau = 1, or all tau = 1 with
-// boxes the moment kernel takes (nx % 4 == 0, nx >= tile width + 8)
-// (kBatchMomentElem: all tau = 1, some box not split into 16-byte row chunks: the
-// moment kernel with element copies)
-// (kBatchRow / kBatchRowAny: the row kernel, all boxes with aligned rows / any)
+// batch kernel modes: the pipelined kernel for lattices with mixed tau or all tau = 1,
+// the moment kernel (all tau = 1) with row chunks (nx % 4 == 0, nx >= tile width + 8)
+// or with element copies, the row kernel with all rows aligned or any rows
 enum BatchMode : int { kBatchMixedTau = 0, kBatchUnitTau = 1, kBatchMoment = 2, kBatchMomentElem = 3,
                        kBatchRow = 4, kBatchRowAny = 5 };
+constexpr int kBatchModes = 6;
 constexpr bool batch_mode_row(int mode) { return mode == kBatchRow || mode == kBatchRowAny; }
 // rows of a batch item of this box under the row kernel: as many as a CTA holds (all
 // items of a launch share one split of the warps), evened out over the box; 0 where
@@ -273,6 +272,43 @@ inline TileCfg batch_tile(int prec, int stencil, int mode) {
   t.kind = mode == kBatchMoment ? 5 : (mode == kBatchMomentElem ? 6 : 1);
   return t;
 }
+// whether the kernel of a batch mode takes a lattice
+inline bool batch_mode_takes(int prec, int stencil, int mode, int nx, int ny, int nz, double tau) {
+  if (mode == kBatchMixedTau) return prec != kF16;
+  if (tau != 1.0) return false;
+  switch (mode) {
+    case kBatchUnitTau:
+    case kBatchMomentElem: return prec != kF16;
+    // (a tile's staged row, 16-byte chunks of the box's row, wraps in x at most once)
+    case kBatchMoment: return nx % (prec == kF16 ? 8 : 4) == 0 && nx >= (prec == kF16 ? 48 : batch_tile(prec, stencil, mode).bx + 8);
+    case kBatchRow: return nx % (prec == kF16 ? 8 : 4) == 0 && row_batch_rows(prec, stencil, nx, ny, nz) > 0;
+    case kBatchRowAny: return prec == kF32 && row_batch_rows(prec, stencil, nx, ny, nz) > 0;
+  }
+  return false;
+}
+// The modes that take a set of lattices, and the one it gets: the row kernel where it
+// takes every box and the lattices together are worth its few large items (a launch of
+// 152 CTAs; below 190000 nodes in all the tile kernels' many small CTAs are faster).
+struct BatchMix {
+  int prec, stencil;
+  bool all[kBatchModes] = {true, true, true, true, true, true};
+  double nodes = 0.0;
+  void add(int nx, int ny, int nz, double tau) {
+    for (int m = 0; m < kBatchModes; ++m) all[m] = all[m] && batch_mode_takes(prec, stencil, m, nx, ny, nz, tau);
+    nodes += (double)nx * ny * nz;
+  }
+  bool takes(int mode) const { return mode >= 0 && mode < kBatchModes && all[mode]; }
+  int mode() const {
+    if (nodes >= 190000.0)
+      for (int m : {kBatchRow, kBatchRowAny})
+        if (all[m]) return m;
+    for (int m : {kBatchMoment, kBatchMomentElem, kBatchMixedTau})
+      if (all[m]) return m;
+    return kBatchMoment;
+  }
+  // the modes that the batch autotuner times: the mix's own, and the tile kernels at tau = 1
+  bool candidate(int m) const { return m == mode() || (all[m] && m >= kBatchUnitTau && m <= kBatchMomentElem); }
+};
 cudaError_t launch_row_batch_any(int prec, bool aligned, const BatchEntry* table, const BatchHeader* hdr, int step,
                                  bool prepare, int* grid, cudaStream_t s);
 // items of one lattice in a batch launch of this mode, z chunks of zc planes; *rows as
