@@ -160,6 +160,12 @@ __device__ __forceinline__ bool positive_finite_bits(double v) {
   return (unsigned)hi < 0x7ff00000u && (hi | __double2loint(v)) != 0;
 }
 
+// whether vrcp takes v: below, 1/v or its correction would overflow, above it would be
+// flushed, and of an infinity or zero vrcp makes NaN where the division makes 0 or an infinity
+__device__ __forceinline__ bool rcp_range_bits(double v) {   // 2^-1000 <= |v| < 2^1000
+  return (unsigned)((__double2hiint(v) & 0x7fffffff) - 0x01700000) < 0x7e700000u - 0x01700000u;
+}
+
 // minimum-image displacement of coordinate X from the centre node n/2; the plane at
 // exactly half the box (even sizes) is both images and counts as 0
 __device__ __forceinline__ int centre_displacement(int X, int n) {
@@ -251,7 +257,7 @@ lattice_kernel(LatticeDesc d, int zchunk, ObsArgs oa) {
         for (int i = 0; i < Q; ++i) gd[i] = widen(g[i]);
         double dnd, jxd, jyd, jzd;
         moments(gd, dnd, jxd, jyd, jzd);
-        const double nd = d.n0 + dnd, inv_n = vrcp(nd);
+        const double nd = d.n0 + dnd, inv_n = rcp_range_bits(nd) ? vrcp(nd) : 1.0 / nd;
         const double uxd = __fma_rn(0.5, widen(Fx), jxd) * inv_n;
         const double uyd = __fma_rn(0.5, widen(Fy), jyd) * inv_n;
         const double uzd = __fma_rn(0.5, widen(Fz), jzd) * inv_n;

@@ -30,10 +30,12 @@ template <> struct Lane<float2> {
   static __device__ __forceinline__ float2 all(float x) { return make_float2(x, x); }
 };
 
-// 1/n to within an ulp: the hardware's approximate reciprocal (relative error e
-// of 2^-23 in FP32, about 2^-20 in FP64) and one correction, of first order in
-// FP32 (e^2) and second order in FP64 (e^3).  An IEEE division costs three times
-// the instructions.
+// 1/n to within an ulp of the division: the hardware's approximate reciprocal y
+// (relative error e = 1 - n y of 2^-23 in FP32, about 2^-20 in FP64) and one
+// Newton-Raphson correction y (1 + e) in FP32 (the rest is e^2), the third-order one
+// y (1 + e + e^2) in FP64 (the rest is e^3).  An IEEE division costs three times the
+// instructions.  For normal n with a normal reciprocal; of 0 and of infinities it
+// makes NaN, as the collision of such a node does anyhow (n u.u is 0 times infinity).
 __device__ __forceinline__ float vrcp(float n) {
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(n));
