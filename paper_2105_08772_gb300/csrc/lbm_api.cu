@@ -54,6 +54,8 @@ struct lbm_ctx {
   int graph_len;
   lbm_obs last;
   int have_last;
+  RowPlan rows;               // the row kernel's cut of the box (plan_rows, at the first step)
+  bool rows_planned;
   TmaMaps tma;                // tensor maps of pop[0] / pop[1] for the TMA step kernel (kind 7)
   char err[512];
 };
@@ -169,6 +171,7 @@ LatticeDesc desc_of(const lbm_ctx* c, int src_buf) {
   d.err = c->err_dev;
   d.aux = c->aux;
   d.tma = c->tma.ok ? &c->tma : nullptr;
+  d.rows = c->rows.ok ? &c->rows : nullptr;
   set_float_params(d);
   return d;
 }
@@ -394,7 +397,23 @@ lbm_status prepare_kernels(lbm_ctx* c) {
   return LBM_OK;
 }
 
+// The row kernel's cut of this box, searched once per lattice (up to a millisecond for
+// flat boxes) and not at its creation, since batches and groups have no use for it.
+lbm_status plan_rows(lbm_ctx* c) {
+  if (c->rows_planned) return LBM_OK;
+  if (c->stencil == 4 && c->tau == 1.0) {
+    int dev = 0, sms = 0;
+    LBM_CUDA(c, cudaGetDevice(&dev));
+    LBM_CUDA(c, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    c->rows = row_plan(c->prec, c->box.nx, c->box.ny, c->box.nz, sms);
+  }
+  c->rows_planned = true;
+  return LBM_OK;
+}
+
 lbm_status launch_steps_eager(lbm_ctx* c, long long n, cudaStream_t s) {
+  const lbm_status planned = plan_rows(c);
+  if (planned != LBM_OK) return planned;
   ObsArgs oa{};
   for (long long k = 0; k < n; ++k) {
     LatticeDesc d = desc_of(c, c->cur);
@@ -583,6 +602,8 @@ lbm_status lbm_create(lbm_box box, double tau, double G, lbm_eos eos, int stenci
   c->obs_zchunk = default_obs_zchunk(box);
   c->graph[0] = c->graph[1] = nullptr;
   c->graph_len = 128;
+  c->rows = RowPlan{};
+  c->rows_planned = false;
   cudaError_t e = cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking);
   if (e != cudaSuccess) {
     delete c;

@@ -143,6 +143,7 @@ struct LatticeDesc {
   int* err;             // device flag set by a kernel whose bounded wait ran out (may be null)
   void* aux;            // one plane of psi between the two passes of a step (null: FP16)
   const void* tma;      // host: the lattice's TMA tensor maps (TmaMaps) or null; kernels ignore it
+  const void* rows;     // host: the lattice's cut for the row kernel (RowPlan) or null; kernels ignore it
 };
 
 // The float copies of a descriptor's double parameters; call after setting them.

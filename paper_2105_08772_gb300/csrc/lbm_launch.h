@@ -158,7 +158,7 @@ constexpr long long row_min_nodes(int prec, bool aligned) {
 struct RowPlan {
   bool ok;
   bool aligned;   // rows are whole 16-byte pieces
-  int items;
+  int items, grid;
   RowCfg cfg;
 };
 
@@ -176,10 +176,10 @@ struct RowPlan {
 // (9%).
 inline RowPlan row_plan(int prec, int nx, int ny, int nz, int sms) {
   constexpr int R = 1;   // E4 (E6 in rows: 256^3 730 us, the two passes 545)
-  RowPlan best{false, false, 0, {0, 0, 0, 0}};
+  RowPlan best{false, false, 0, 0, {0, 0, 0, 0}};
   const int es = prec == kF16 ? 2 : 4, ve = 16 / es;
   const bool aligned = nx % ve == 0;
-  if (prec == kF64 || nx < 2 * R + 1 || ny < 2 * R + 1 || nz < 2 * R + 1) return best;
+  if (prec == kF64 || (prec == kF16 && !aligned) || nx < 2 * R + 1 || ny < 2 * R + 1 || nz < 2 * R + 1) return best;
   if ((long long)nx * ny * nz < row_min_nodes(prec, aligned)) return best;
   const RowCaps caps = row_caps(prec);
   const double bytes = (double)nx * ny * nz * 38.0 * es;
@@ -198,18 +198,19 @@ inline RowPlan row_plan(int prec, int nx, int ny, int nz, int sms) {
     const int nc = (wc + turns - 1) / turns, cols = (ny + by - 1) / by;
     const double lat_d = 1.15 * scale, lat_c = 0.134 * turns * scale + 0.285;
     const double plane = (lat_d > lat_c ? lat_d : lat_c) + 0.0282 * (wd + 1.07 * wc) * scale;
-    for (int chunks = 1; chunks <= nz; ++chunks) {
-      const int zc = (nz + chunks - 1) / chunks;
-      if (chunks > 1 && zc == (nz + chunks - 2) / (chunks - 1)) continue;
+    for (int chunks = 1, zc = nz;; chunks = (nz + zc - 2) / (zc - 1)) {   // the next with fewer planes
+      zc = (nz + chunks - 1) / chunks;
       const long long items = (long long)cols * ((nz + zc - 1) / zc), rounds = (items + sms - 1) / sms;
       const double sm = rounds * ((zc + 2 * R) * plane + 0.3);
       double mem = bytes / 9e6;
       if (bytes > 2.3e8) mem = bytes / 6.55e6 * (1.0 + (bytes > 5e8 ? 1.0 : 2.0) * R / zc);
       if (bytes > 5e8 && prec == kF32) mem *= 1.0 + 0.02 * (chunks - 2);
       const double a = sm * sm * sm, b = mem * mem * mem, t = a * a + b * b;   // (sm^6 + mem^6): rises with the time
-      if (best.ok && t >= best_t) continue;
-      best_t = t;
-      best = RowPlan{true, aligned, (int)items, {by, zc, nd * 32, nc * 32}};
+      if (!best.ok || t < best_t) {
+        best_t = t;
+        best = RowPlan{true, aligned, (int)items, (int)(items < sms ? items : sms), {by, zc, nd * 32, nc * 32}};
+      }
+      if (zc == 1) break;
     }
   }
   return best;
@@ -233,7 +234,7 @@ inline bool split_applies(int prec, int stencil, bool unit_tau, long long nodes)
   return nodes <= 1500000;
 }
 
-// The whole-row kernel (F32, F16; E4, tau = 1) where its plan has a cut of the box;
+// The whole-row kernel (F32, F16; E4, tau = 1) where the lattice has a plan (d.rows);
 // cudaErrorNotSupported (nothing launched) where it has not.
 cudaError_t launch_row_any(int prec, const LatticeDesc& d, bool prepare, cudaStream_t s);
 

@@ -5,47 +5,35 @@
 
 namespace lbm {
 
+// Launched with programmatic serialisation (the next step's CTAs take over SM by SM:
+// 128^3 58.5 -> 56.2 us, 64^3 17.8 -> 15.2 us when it came in).
 template <int P, bool ALIGNED>
-static cudaError_t launch_row_shape(const LatticeDesc& d, const RowPlan& r, int sms, bool prepare, cudaStream_t s) {
+static cudaError_t launch_row_shape(const LatticeDesc& d, const RowPlan* r, cudaStream_t s) {
   using Sh = RowShape<P, 4>;
   auto kern = lattice_row_kernel<Sh, ALIGNED>;
-  if (prepare)
+  if (!r)   // prepare
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::smem_bytes);
-  const int grid = r.items < sms ? r.items : sms;
   // every other step walks the planes downwards: what the last step wrote last is
   // read first, from L2 (128^3 54.1 -> 53.1 us, 192^3 170.4 -> 169.5, 157^3 100.5 -> 101.5)
   const int flip = reinterpret_cast<uintptr_t>(d.src) > reinterpret_cast<uintptr_t>(d.dst);
-  return launch_step_kernel(kern, grid, r.cfg.nd + r.cfg.nc + 32, Sh::smem_bytes, s, true, d, r.cfg, flip);
+  return launch_step_kernel(kern, r->grid, r->cfg.nd + r->cfg.nc + 32, Sh::smem_bytes, s, true, d, r->cfg, flip);
 }
 
-// The whole-row kernel where the plan has a cut; cudaErrorNotSupported (nothing
-// launched) where it has not.  One CTA per SM; launched with programmatic
-// serialisation (the next step's CTAs take over SM by SM: 128^3 58.5 -> 56.2 us, 64^3
-// 17.8 -> 15.2 us when it came in).
+// The whole-row kernel by the lattice's plan; cudaErrorNotSupported (nothing launched)
+// where it has none.  One CTA per SM.
 template <int P>
 static cudaError_t launch_row(const LatticeDesc& d, bool prepare, cudaStream_t s) {
-  static int sms = 0;
-  if (prepare || sms == 0) {
-    int dev = 0, n = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = launch_row_shape<P, true>(d, RowPlan{}, 0, true, s);
+  const RowPlan* r = static_cast<const RowPlan*>(d.rows);
+  if (prepare) {
+    cudaError_t e = launch_row_shape<P, true>(d, nullptr, s);
     if constexpr (P != kF16)
-      if (e == cudaSuccess) e = launch_row_shape<P, false>(d, RowPlan{}, 0, true, s);
-    if (e == cudaSuccess) sms = n;
-    if (e != cudaSuccess || prepare) return e;
+      if (e == cudaSuccess) e = launch_row_shape<P, false>(d, nullptr, s);
+    return e;
   }
-  // the last box's plan: a step-by-step caller would search it (about 20 us) each time
-  static thread_local int box[4] = {0, 0, 0, 0};
-  static thread_local RowPlan r;
-  if (box[0] != d.nx || box[1] != d.ny || box[2] != d.nz || box[3] != sms) {
-    r = row_plan(P, d.nx, d.ny, d.nz, sms);
-    box[0] = d.nx; box[1] = d.ny; box[2] = d.nz; box[3] = sms;
-  }
-  if (!r.ok) return cudaErrorNotSupported;
-  if (r.aligned) return launch_row_shape<P, true>(d, r, sms, false, s);
+  if (!r || !r->ok) return cudaErrorNotSupported;
+  if (r->aligned) return launch_row_shape<P, true>(d, r, s);
   if constexpr (P == kF16) return cudaErrorNotSupported;
-  else return launch_row_shape<P, false>(d, r, sms, false, s);
+  else return launch_row_shape<P, false>(d, r, s);
 }
 
 template <int P, bool ALIGNED>

@@ -15,3 +15,19 @@ extern "C" int rule_batch_mix(int prec, int stencil, int n, const int* boxes, co
   }
   return m.mode();
 }
+
+// out: ok, aligned, items, grid, by, zc, density threads, collision threads
+extern "C" void rule_row_plan(int prec, int nx, int ny, int nz, int sms, int* out) {
+  const RowPlan r = row_plan(prec, nx, ny, nz, sms);
+  const int v[8] = {r.ok, r.aligned, r.items, r.grid, r.cfg.by, r.cfg.zc, r.cfg.nd, r.cfg.nc};
+  for (int k = 0; k < 8; ++k) out[k] = v[k];
+}
+extern "C" int rule_row_batch_rows(int prec, int stencil, int nx, int ny, int nz) {
+  return row_batch_rows(prec, stencil, nx, ny, nz);
+}
+// out: slot, mcap, kd, threads of a CTA at most, density and collision warps of a batch CTA
+extern "C" void rule_row_caps(int prec, int* out) {
+  const RowCaps c = row_caps(prec);
+  const int v[6] = {c.slot, c.mcap, c.kd, kRowThreads, kRowBatchDensityWarps, kRowBatchCollideWarps};
+  for (int k = 0; k < 6; ++k) out[k] = v[k];
+}
