@@ -411,13 +411,16 @@ lbm_status plan_rows(lbm_ctx* c) {
   return LBM_OK;
 }
 
-lbm_status launch_steps_eager(lbm_ctx* c, long long n, cudaStream_t s) {
+// n steps, launched on the lattice's stream or captured on its private one
+lbm_status launch_steps(lbm_ctx* c, long long n, cudaStream_t s) {
   const lbm_status planned = plan_rows(c);
   if (planned != LBM_OK) return planned;
   ObsArgs oa{};
+  TileCfg cfg = c->step_cfg;
+  cfg.eager = s != c->cap_stream;
   for (long long k = 0; k < n; ++k) {
     LatticeDesc d = desc_of(c, c->cur);
-    LBM_CUDA(c, launch_lattice(c->prec, c->stencil, kModeStep, d, c->step_cfg, oa, s));
+    LBM_CUDA(c, launch_lattice(c->prec, c->stencil, kModeStep, d, cfg, oa, s));
     c->cur ^= 1;
   }
   return LBM_OK;
@@ -429,7 +432,7 @@ lbm_status ensure_graph(lbm_ctx* c) {
   cudaGraph_t g = nullptr;
   LBM_CUDA(c, cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
   const int cur0 = c->cur;
-  lbm_status st = launch_steps_eager(c, c->graph_len, c->cap_stream);
+  lbm_status st = launch_steps(c, c->graph_len, c->cap_stream);
   c->cur = cur0;   // graph_len is even; capture does not advance the state
   cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
   if (st != LBM_OK) {
@@ -739,7 +742,7 @@ lbm_status lbm_step(lbm_ctx* c, long long n) {
     n -= c->graph_len;
     c->steps += c->graph_len;
   }
-  lbm_status st = launch_steps_eager(c, n, c->stream);
+  lbm_status st = launch_steps(c, n, c->stream);
   if (st != LBM_OK) return st;
   c->steps += n;
   return LBM_OK;
@@ -1007,10 +1010,10 @@ lbm_status lbm_autotune(lbm_ctx* c, int reps, long long* choice) {
   lbm_status st = LBM_OK;
   for (const TileCfg& t : step_candidates(c)) {
     c->step_cfg = t;
-    st = launch_steps_eager(c, 2, c->stream);
+    st = launch_steps(c, 2, c->stream);
     if (st != LBM_OK) break;
     cudaEventRecord(e0, c->stream);
-    st = launch_steps_eager(c, reps, c->stream);
+    st = launch_steps(c, reps, c->stream);
     if (st != LBM_OK) break;
     cudaEventRecord(e1, c->stream);
     cudaError_t e = cudaEventSynchronize(e1);

@@ -421,17 +421,13 @@ static cudaError_t dispatch_lattice(int stencil, int mode, const LatticeDesc& d,
     if (stencil == 4) return dispatch_tma<P, 4>(d, c, s);
     return cudaErrorInvalidValue;
   }
-  // kinds 5 and 6 with a launcher-chosen z chunk: the row kernel where it has a plan,
-  // the two passes where they are the fastest (split_applies)
-  if (mode == kModeStep && (c.kind == 5 || c.kind == 6) && c.zchunk == 0 && !c.prepare) {
+  if (mode == kModeStep && !c.prepare) {
+    const StepRoute route = step_route(P, stencil, d, c);
     if constexpr (P != kF64)
-      if (stencil == 4 && d.omega == 1.0 && c.bx == 32 && c.by == 8) {
-        const cudaError_t e = launch_row_any(P, d, false, s);
-        if (e != cudaErrorNotSupported) return e;
-      }
+      if (route == kRouteRow) return launch_row_any(P, d, false, s);
     if constexpr (P != kF16) {
       using T = typename Storage<P>::T;
-      if (d.aux && split_applies(P, stencil, d.omega == 1.0, d.plane)) {
+      if (route == kRouteSplit) {
         if (stencil == 4) return launch_split<T, 4>(d, s);
         if (stencil == 6) return launch_split<T, 6>(d, s);
         if (stencil == 8) return launch_split<T, 8>(d, s);

@@ -23,6 +23,7 @@ struct TileCfg {
   int kind = 0;
   int depth = 1;
   bool prepare = false;
+  bool eager = false;   // the step is launched by itself, not captured for replays
 };
 
 // TMA tensor maps of both population buffers of one lattice (host side; kind 7):
@@ -232,6 +233,31 @@ inline long long lattice_grid_ctas(const LatticeDesc& d, TileCfg cfg) {
 inline bool split_applies(int prec, int stencil, bool unit_tau, long long nodes) {
   if (prec == kF64 || stencil == 6 || (stencil == 8 && unit_tau)) return true;
   return nodes <= 1500000;
+}
+
+// FP32 steps launched one by one, where a second launch costs more than the two passes
+// gain: boxes with at most one plane of one tile for each SM (32 x 8 tiles, E6 and E8
+// 32 x 4).  us a step over 100 launches, one launch against two: E4 8^3 to 32^3 6.2 /
+// 8.2, 100x3x3 6.2 / 8.2, 48x48x12 8.2 / 8.2, tau 0.8 28^3 7.2 / 8.2; past the line
+// 33^3 10.4 / 8.2, 3x100x100 14.7 / 8.2.  E6 and E8 gain in strips alone: 100x5x5 8.2 /
+// 10.3, but 24^3 8.2 / 8.2 and a single step of 8^3 16.2 / 14.7.  (In a replayed graph
+// the launches cost less and the two passes win: 8^3 4.1 / 2.8.)
+inline bool eager_one_launch(int prec, int stencil, int nx, int ny, int nz) {
+  const int by = stencil == 4 ? 8 : 4;
+  const long long planes = (long long)((nx + 31) / 32) * ((ny + by - 1) / by) * nz;
+  return prec == kF32 && planes <= 152 && (stencil == 4 || nx >= 64);
+}
+
+// What a step of this configuration runs: a tile kernel by its own name, or, behind
+// kinds 5 and 6 with a launcher-chosen z chunk, the row kernel where the lattice has a
+// plan (d.rows), the two passes where they are faster.
+enum StepRoute : int { kRouteTile = 0, kRouteRow = 1, kRouteSplit = 2 };
+inline StepRoute step_route(int prec, int stencil, const LatticeDesc& d, const TileCfg& c) {
+  if ((c.kind != 5 && c.kind != 6) || c.zchunk != 0) return kRouteTile;
+  const bool unit_tau = d.omega == 1.0;
+  if (stencil == 4 && unit_tau && c.bx == 32 && c.by == 8 && d.rows) return kRouteRow;
+  if (!d.aux || !split_applies(prec, stencil, unit_tau, d.plane)) return kRouteTile;
+  return c.eager && eager_one_launch(prec, stencil, d.nx, d.ny, d.nz) ? kRouteTile : kRouteSplit;
 }
 
 // The whole-row kernel (F32, F16; E4, tau = 1) where the lattice has a plan (d.rows);

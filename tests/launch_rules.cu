@@ -31,3 +31,20 @@ extern "C" void rule_row_caps(int prec, int* out) {
   const int v[6] = {c.slot, c.mcap, c.kd, kRowThreads, kRowBatchDensityWarps, kRowBatchCollideWarps};
   for (int k = 0; k < 6; ++k) out[k] = v[k];
 }
+
+// the route of a default step (kind 5 or 6, launcher-chosen z chunk), with a psi plane
+extern "C" int rule_step_route(int prec, int stencil, int unit_tau, int nx, int ny, int nz, int eager) {
+  const RowPlan r = row_plan(prec, nx, ny, nz, 152);
+  LatticeDesc d{};
+  d.nx = nx;
+  d.ny = ny;
+  d.nz = nz;
+  d.plane = (long long)nx * ny * nz;
+  d.omega = unit_tau ? 1.0 : 1.25;
+  d.aux = prec == kF16 ? nullptr : &d;
+  d.rows = r.ok && unit_tau && stencil == 4 ? &r : nullptr;
+  TileCfg c{32, stencil == 4 ? 8 : 4, 0};
+  c.kind = 5;
+  c.eager = eager != 0;
+  return step_route(prec, stencil, d, c);
+}

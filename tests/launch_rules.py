@@ -56,3 +56,8 @@ def row_caps(prec):
     out = (ctypes.c_int * 6)()
     compile_so("launch_rules.cu").rule_row_caps(PREC[prec], out)
     return dict(zip(("slot", "mcap", "kd", "threads", "batch_nd", "batch_nc"), out))
+
+
+def step_route(prec, box, stencil=4, unit_tau=True, eager=False):
+    """what a default step runs: 0 a tile kernel, 1 the row kernel, 2 the two passes"""
+    return compile_so("launch_rules.cu").rule_step_route(PREC[prec], stencil, int(unit_tau), *box, int(eager))
