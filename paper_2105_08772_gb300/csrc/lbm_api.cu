@@ -426,6 +426,16 @@ lbm_status launch_steps(lbm_ctx* c, long long n, cudaStream_t s) {
   return LBM_OK;
 }
 
+constexpr long long kGraphFrom = 128;   // calls of fewer steps are launched one by one
+lbm_status choose_graph_len(lbm_ctx* c) {
+  const lbm_status planned = plan_rows(c);
+  if (planned != LBM_OK) return planned;
+  const int len = steps_per_graph(step_route(c->prec, c->stencil, desc_of(c, 0), c->step_cfg));
+  if (len != c->graph_len) drop_graphs(c);
+  c->graph_len = len;
+  return LBM_OK;
+}
+
 lbm_status ensure_graph(lbm_ctx* c) {
   const int p = c->cur;
   if (c->graph[p]) return LBM_OK;
@@ -735,14 +745,19 @@ lbm_status lbm_step(lbm_ctx* c, long long n) {
   LBM_CHECK_CTX(c);
   LBM_CHECK_INIT(c);
   if (n < 0) return fail(c, LBM_EINVAL, "n must be >= 0");
-  while (n >= c->graph_len) {
-    lbm_status st = ensure_graph(c);
+  lbm_status st;
+  if (n >= kGraphFrom) {
+    st = choose_graph_len(c);
     if (st != LBM_OK) return st;
-    LBM_CUDA(c, cudaGraphLaunch(c->graph[c->cur], c->stream));
-    n -= c->graph_len;
-    c->steps += c->graph_len;
+    while (n >= c->graph_len) {
+      st = ensure_graph(c);
+      if (st != LBM_OK) return st;
+      LBM_CUDA(c, cudaGraphLaunch(c->graph[c->cur], c->stream));
+      n -= c->graph_len;
+      c->steps += c->graph_len;
+    }
   }
-  lbm_status st = launch_steps(c, n, c->stream);
+  st = launch_steps(c, n, c->stream);
   if (st != LBM_OK) return st;
   c->steps += n;
   return LBM_OK;

@@ -260,6 +260,13 @@ inline StepRoute step_route(int prec, int stencil, const LatticeDesc& d, const T
   return c.eager && eager_one_launch(prec, stencil, d.nx, d.ny, d.nz) ? kRouteTile : kRouteSplit;
 }
 
+// Steps of a captured graph: 128 kernels of it, since a lattice captures its graph anew
+// after each initialisation (the storage shift is among the kernels' parameters).  us a
+// step, initialisation and 128 steps, 128 steps of two passes a graph against 64: 16^3
+// 8.2 / 6.3, 64^3 19.5 / 17.6, tau 0.8 96^3 58.7 / 56.9, FP64 32^3 18.6 / 16.6; a run of
+// 2048 steps takes the same.
+constexpr int steps_per_graph(StepRoute route) { return route == kRouteSplit ? 64 : 128; }
+
 // The whole-row kernel (F32, F16; E4, tau = 1) where the lattice has a plan (d.rows);
 // cudaErrorNotSupported (nothing launched) where it has not.
 cudaError_t launch_row_any(int prec, const LatticeDesc& d, bool prepare, cudaStream_t s);

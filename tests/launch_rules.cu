@@ -48,3 +48,4 @@ extern "C" int rule_step_route(int prec, int stencil, int unit_tau, int nx, int 
   c.eager = eager != 0;
   return step_route(prec, stencil, d, c);
 }
+extern "C" int rule_steps_per_graph(int route) { return steps_per_graph((StepRoute)route); }

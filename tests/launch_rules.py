@@ -61,3 +61,7 @@ def row_caps(prec):
 def step_route(prec, box, stencil=4, unit_tau=True, eager=False):
     """what a default step runs: 0 a tile kernel, 1 the row kernel, 2 the two passes"""
     return compile_so("launch_rules.cu").rule_step_route(PREC[prec], stencil, int(unit_tau), *box, int(eager))
+
+
+def steps_per_graph(route):
+    return compile_so("launch_rules.cu").rule_steps_per_graph(route)

@@ -22,3 +22,11 @@ def test_small_fp32_steps_take_one_launch_unless_captured(box, unit_tau):
 def test_where_the_line_lies(prec, box, stencil, route):
     assert launch_rules.step_route(prec, box, stencil, eager=True) == route
     assert launch_rules.step_route(prec, box, stencil) == SPLIT
+
+
+def test_a_graph_holds_128_kernels():
+    """A graph is captured anew after every initialisation, so two kernels a step do not
+    make it twice as long."""
+    for box, route in (((64, 64, 64), SPLIT), ((128, 128, 128), ROW)):
+        assert launch_rules.step_route("f32", box) == route
+        assert launch_rules.steps_per_graph(route) * (2 if route == SPLIT else 1) == 128
