@@ -386,7 +386,11 @@ lbm_status prepare_kernels(lbm_ctx* c) {
   // outside any stream capture
   LatticeDesc d = desc_of(c, 0);
   ObsArgs oa{};
+  TileCfg last{0, 0, 0, -1, 0};
   for (const TileCfg& t : step_candidates(c)) {
+    // candidates that differ in their z chunk alone come one after another and are one kernel
+    if (t.kind == last.kind && t.bx == last.bx && t.by == last.by && t.depth == last.depth) continue;
+    last = t;
     TileCfg p = t;
     p.prepare = true;
     LBM_CUDA(c, launch_lattice(c->prec, c->stencil, kModeStep, d, p, oa, c->stream));
