@@ -4,6 +4,7 @@
 
 #include <cuda.h>
 #include <cuda_runtime.h>
+#include <math.h>
 
 #include "lbm_common.cuh"
 #include "lbm_kernels.cuh"
@@ -151,7 +152,7 @@ constexpr RowCaps row_caps(int prec) {
 // faster and have more in flight.  us, rows against the other: F32 aligned rows 64^3
 // 11.4 / 9.8, 72^3 12.4 / 12.6, 96^3 22.1 / 26.2; unaligned 70x71x72 15.7 / 11.7, 97^3
 // 31.3 / 27.3, 105^3 36.5 / 35.5, 113^3 43.9 / 48.3; F16 64^3 rows, 48^3 the moment
-// kernel.
+// kernel.  (row_pays leaves out more, by shape.)
 constexpr long long row_min_nodes(int prec, bool aligned) {
   return prec == kF16 ? 190000 : aligned ? 350000 : 1200000;
 }
@@ -162,6 +163,37 @@ struct RowPlan {
   int items, grid;
   RowCfg cfg;
 };
+
+// Whether a cut is expected to beat what the box runs otherwise.  Its time is that of
+// row_plan, a start of 3 us (FP32), and at least the copies of each plane: 19 at 0.045 us
+// each and their bytes at 54 per clock, several times as many where the blocks wrap
+// around a short box in y (64x3x5000 67 us, the moment kernel 38).  One-row FP16 items
+// (rows past 576 nodes, densities formed three times) count for a third more.  The
+// others: the two passes (FP32 up to 1.5 million nodes) 28 nodes a nanosecond (30 in a
+// replayed graph, but two launches where steps are launched one by one: 64x64x100 13.2 us
+// in rows, 13.5, and 13.7 against 18.6 launched singly); the moment kernel 27 (aligned
+// rows), 23 (any rows; odd boxes), in FP32 its last tile of a row counted whole.
+// Measured on 456 boxes of 3 to 1389 rows and 3 to 31250 planes: the choice is 0.4% off
+// the faster kernel on the mean, 13% at most; with the row kernel wherever it has a cut it
+// was 9% on the mean and up to 3.5 times (us, row kernel / other: 33x3x20000 502 / 144,
+// 449x80x80 142 / 108, 96x16x4461 240 / 194, F16 600x64x64 64.7 / 54.8).
+inline bool row_pays(int prec, int nx, int ny, int nz, int sms, const RowPlan& r, double plane, double mem) {
+  constexpr int R = 1;
+  const double nodes = (double)nx * ny * nz;
+  const int by = r.cfg.by, zc = r.cfg.zc, es = prec == kF16 ? 2 : 4;
+  const int wraps = by + 2 * R <= ny && ny >= 3 * by ? 1 : (by + 2 * R <= 2 * ny ? 2 : 3);
+  const double copies = 19.0 * (0.045 * wraps + (double)(by + 2 * R) * nx * es / 54.0 / 1900.0);
+  const double rounds = (r.items + sms - 1) / sms;
+  const double sm = rounds * ((zc + 2 * R) * (plane > copies ? plane : copies) + 0.3) + (prec == kF16 ? 0.0 : 3.0);
+  const double a = sm * sm * sm, b = mem * mem * mem;
+  double t = cbrt(sqrt(a * a + b * b));
+  if (prec == kF16) {
+    if (by == 1) t *= 1.35;
+    return t < nodes / 27e3;
+  }
+  if (nodes <= 1.5e6) return t < nodes / 28e3;
+  return t < (double)((nx + 31) / 32 * 32) * ny * nz / (r.aligned ? 27e3 : 23e3);
+}
 
 // The cut with the least expected time, or ok = false where no item fits (rows too
 // long) or the box is too small for the copies' wrap.
@@ -174,7 +206,8 @@ struct RowPlan {
 // The constants (microseconds) were
 // fitted to 2300 measured cuts of 28 boxes, 24^3 to 256^3, odd and ragged ones among
 // them: the plan's choice is within 4% of the best cut of each, but for two FP16 boxes
-// (9%).
+// (128^3 9%, 160^3 10%).  There is no plan where the other kernel is expected to be
+// faster (row_pays).
 inline RowPlan row_plan(int prec, int nx, int ny, int nz, int sms) {
   constexpr int R = 1;   // E4 (E6 in rows: 256^3 730 us, the two passes 545)
   RowPlan best{false, false, 0, 0, {0, 0, 0, 0}};
@@ -185,7 +218,7 @@ inline RowPlan row_plan(int prec, int nx, int ny, int nz, int sms) {
   const RowCaps caps = row_caps(prec);
   const double bytes = (double)nx * ny * nz * 38.0 * es;
   const double scale = (aligned ? 1.0 : 1.42) * (prec == kF16 ? 0.9 : 1.0);
-  double best_t = 0.0;
+  double best_t = 0.0, best_plane = 0.0, best_mem = 0.0;
   for (int by = 1; by <= ny; ++by) {
     const long long nodes = (long long)(by + 2 * R) * nx, inner = (long long)by * nx;
     if (nodes > caps.slot - 4 * ve || inner > caps.mcap) break;
@@ -209,11 +242,14 @@ inline RowPlan row_plan(int prec, int nx, int ny, int nz, int sms) {
       const double a = sm * sm * sm, b = mem * mem * mem, t = a * a + b * b;   // (sm^6 + mem^6): rises with the time
       if (!best.ok || t < best_t) {
         best_t = t;
+        best_plane = plane;
+        best_mem = mem;
         best = RowPlan{true, aligned, (int)items, (int)(items < sms ? items : sms), {by, zc, nd * 32, nc * 32}};
       }
       if (zc == 1) break;
     }
   }
+  if (best.ok && !row_pays(prec, nx, ny, nz, sms, best, best_plane, best_mem)) best.ok = false;
   return best;
 }
 

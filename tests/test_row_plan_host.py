@@ -83,3 +83,23 @@ def test_a_long_box_is_planned_quickly():
     t0 = time.perf_counter()
     launch_rules.row_plan("f32", (8, 8, 2000000))
     assert time.perf_counter() - t0 < 0.01
+
+
+@pytest.mark.parametrize("prec,box,planned", [
+    # blocks of few rows wrap around the box in y: three copies where one is usual
+    ("f32", (64, 3, 5000), False), ("f32", (33, 3, 20000), False), ("f32", (32, 8, 8593), False),
+    ("f32", (400, 6, 916), True), ("f32", (64, 24, 1432), True), ("f16", (64, 4, 8593), False),
+    # items of one row, densities formed three times
+    ("f32", (449, 80, 80), False), ("f32", (450, 64, 64), False), ("f32", (597, 64, 64), False),
+    ("f32", (549, 100, 100), True), ("f32", (512, 100, 100), True), ("f32", (452, 30, 30), False),
+    ("f16", (600, 64, 64), False), ("f16", (640, 20, 16), False), ("f16", (768, 100, 100), True),
+    # ordinary boxes
+    ("f32", (128, 128, 128), True), ("f32", (256, 256, 256), True), ("f32", (157, 157, 157), True),
+    ("f32", (72, 72, 72), True), ("f32", (64, 64, 100), True), ("f32", (96, 96, 96), True), ("f32", (113, 113, 113), True), ("f32", (335, 335, 335), True),
+    ("f32", (335, 41, 90), True), ("f32", (440, 48, 60), True), ("f16", (64, 64, 64), True),
+    ("f16", (128, 128, 128), True), ("f16", (256, 256, 256), True), ("f16", (256, 40, 33), True),
+])
+def test_where_the_row_kernel_pays(prec, box, planned):
+    """Measured on both sides of the line (GB300): the row kernel has a plan only where it is
+    the faster one."""
+    assert (launch_rules.row_plan(prec, box) is not None) == planned
