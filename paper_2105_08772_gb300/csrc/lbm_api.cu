@@ -1491,9 +1491,12 @@ BatchLayout batch_layout(int slots, lbm_box max_box, int stencil, int prec) {
   return L;
 }
 
-// the whole queue as a mix of lattices
+constexpr int kBatchTileChunk = 16;   // planes of a batch's item under the tile kernels
+
+// the whole queue as a mix of lattices, of which the slots hold some at a time
 BatchMix queue_mix(const lbm_batch* b) {
-  BatchMix m{b->prec, b->stencil};
+  const int cap = b->slot_cap > 0 && b->slot_cap < b->slots ? b->slot_cap : b->slots;
+  BatchMix m{b->prec, b->stencil, cap, kBatchTileChunk};
   for (const BatchRun& r : b->runs) m.add(r.box.nx, r.box.ny, r.box.nz, r.tau);
   return m;
 }
@@ -1542,26 +1545,11 @@ lbm_status batch_fill(lbm_batch* b) {
   return LBM_OK;
 }
 
-// One z chunk for all lattices of a launch on `grid` resident CTAs, chosen like the
-// single-lattice launcher's (fewest rounds x planes).
 int common_zchunk(int prec, int stencil, int mode, const std::vector<lbm_ctx*>& ctx, int grid) {
-  const int R = radius_of(stencil);
-  int max_nz = 1, rows = 0;
+  std::vector<MixBox> b;
   for (const lbm_ctx* c : ctx)
-    if (c && c->box.nz > max_nz) max_nz = c->box.nz;
-  int best_zc = max_nz;
-  long long best_cost = -1;
-  for (int zc = 1; zc <= max_nz; ++zc) {
-    long long items = 0;
-    for (const lbm_ctx* c : ctx)
-      if (c) items += batch_items(prec, stencil, mode, c->box.nx, c->box.ny, c->box.nz, zc, &rows);
-    const long long rounds = (items + grid - 1) / grid, cost = rounds * (zc + 2 * R);
-    if (best_cost < 0 || cost <= best_cost) {
-      best_cost = cost;
-      best_zc = zc;
-    }
-  }
-  return best_zc;
+    if (c) b.push_back(MixBox{c->box.nx, c->box.ny, c->box.nz});
+  return lbm::common_zchunk(prec, stencil, mode, b.data(), (int)b.size(), grid);
 }
 
 // table of the active lattices, in slot order, with their global work items
@@ -1570,7 +1558,7 @@ lbm_status batch_upload(lbm_batch* b) {
   long long items = 0;
   // tile kernels: chunks of 16 planes; the row kernel's few large items are evened out
   const int auto_zc = batch_mode_row(b->graph_mode) && b->zchunk == 0 && b->grid > 0
-                          ? common_zchunk(b->prec, b->stencil, b->graph_mode, b->slot_ctx, b->grid) : 16;
+                          ? common_zchunk(b->prec, b->stencil, b->graph_mode, b->slot_ctx, b->grid) : kBatchTileChunk;
   for (int k = 0; k < b->slots; ++k) {
     lbm_ctx* c = b->slot_ctx[k];
     if (!c) continue;
@@ -1974,7 +1962,7 @@ lbm_status lbm_group_create(lbm_ctx* const* ctxs, int n, void* dev_workspace, si
   char* ws = static_cast<char*>(dev_workspace);
   g->table_dev = reinterpret_cast<BatchEntry*>(ws);
   g->hdr_dev = reinterpret_cast<BatchHeader*>(ws + align256(sizeof(BatchEntry) * (size_t)n));
-  BatchMix mix{g->prec, g->stencil};   // kernel mode as for a batch
+  BatchMix mix{g->prec, g->stencil, 0, 0};   // all at a time, the common z chunk
   for (lbm_ctx* c : g->ctx) mix.add(c->box.nx, c->box.ny, c->box.nz, c->tau);
   g->mode = mix.mode();
   cudaError_t e = cudaStreamCreateWithFlags(&g->cap_stream, cudaStreamNonBlocking);

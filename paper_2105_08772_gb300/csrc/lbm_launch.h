@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <vector>
+
 #include "lbm_common.cuh"
 #include "lbm_kernels.cuh"
 
@@ -356,31 +358,6 @@ inline bool batch_mode_takes(int prec, int stencil, int mode, int nx, int ny, in
   }
   return false;
 }
-// The modes that take a set of lattices, and the one it gets: the row kernel where it
-// takes every box and the lattices together are worth its few large items (a launch of
-// 152 CTAs; below 190000 nodes in all the tile kernels' many small CTAs are faster).
-struct BatchMix {
-  int prec, stencil;
-  bool all[kBatchModes] = {true, true, true, true, true, true};
-  double nodes = 0.0;
-  void add(int nx, int ny, int nz, double tau) {
-    for (int m = 0; m < kBatchModes; ++m) all[m] = all[m] && batch_mode_takes(prec, stencil, m, nx, ny, nz, tau);
-    nodes += (double)nx * ny * nz;
-  }
-  bool takes(int mode) const { return mode >= 0 && mode < kBatchModes && all[mode]; }
-  int mode() const {
-    if (nodes >= 190000.0)
-      for (int m : {kBatchRow, kBatchRowAny})
-        if (all[m]) return m;
-    for (int m : {kBatchMoment, kBatchMomentElem, kBatchMixedTau})
-      if (all[m]) return m;
-    return kBatchMoment;
-  }
-  // the modes that the batch autotuner times: the mix's own, and the tile kernels at tau = 1
-  bool candidate(int m) const { return m == mode() || (all[m] && m >= kBatchUnitTau && m <= kBatchMomentElem); }
-};
-cudaError_t launch_row_batch_any(int prec, bool aligned, const BatchEntry* table, const BatchHeader* hdr, int step,
-                                 bool prepare, int* grid, cudaStream_t s);
 // items of one lattice in a batch launch of this mode, z chunks of zc planes; *rows as
 // for BatchEntry::rows
 inline long long batch_items(int prec, int stencil, int mode, int nx, int ny, int nz, int zc, int* rows) {
@@ -393,6 +370,131 @@ inline long long batch_items(int prec, int stencil, int mode, int nx, int ny, in
   const TileCfg t = batch_tile(prec, stencil, mode);
   return chunks * ((nx + t.bx - 1) / t.bx) * ((ny + t.by - 1) / t.by);
 }
+struct MixBox { int nx, ny, nz; };
+// One z chunk for all lattices of a launch on `grid` resident CTAs, chosen like the
+// single-lattice launcher's (fewest rounds x planes).
+inline int common_zchunk(int prec, int stencil, int mode, const MixBox* b, int n, int grid) {
+  const int R = stencil == 4 ? 1 : 2;
+  int max_nz = 1, rows = 0;
+  for (int k = 0; k < n; ++k) max_nz = b[k].nz > max_nz ? b[k].nz : max_nz;
+  int best_zc = max_nz;
+  long long best_cost = -1;
+  for (int zc = 1; zc <= max_nz; ++zc) {
+    long long items = 0;
+    for (int k = 0; k < n; ++k) items += batch_items(prec, stencil, mode, b[k].nx, b[k].ny, b[k].nz, zc, &rows);
+    const long long rounds = (items + grid - 1) / grid, cost = rounds * (zc + 2 * R);
+    if (best_cost < 0 || cost <= best_cost) {
+      best_cost = cost;
+      best_zc = zc;
+    }
+  }
+  return best_zc;
+}
+// Expected microseconds of a step of n lattices (E4, tau = 1), mode kBatchRow or
+// kBatchRowAny.  An item takes 5 us to start (its table entry, its first copies), then
+// each plane a latency and a share for each 64-node piece, as in row_plan with the
+// batch's fixed warps, or its copies (see row_pays) where they take longer.
+inline double batch_row_us(int prec, int mode, const MixBox* b, int n) {
+  constexpr int sms = 152;
+  const int zc = common_zchunk(prec, 4, mode, b, n, sms), es = prec == kF16 ? 2 : 4;
+  const double scale = mode == kBatchRowAny ? 1.64 : 1.0;
+  double total = 0.0, most = 0.0, mem = 0.0;
+  long long items = 0;
+  for (int k = 0; k < n; ++k) {
+    int by = 0;
+    const int z = b[k].nz < zc ? b[k].nz : zc, nx = b[k].nx, ny = b[k].ny;
+    const long long it = batch_items(prec, 4, mode, nx, ny, b[k].nz, z, &by);
+    const int cols = (ny + by - 1) / by, wd = ((by + 2) * nx + 63) / 64, wc = (by * nx + 63) / 64;
+    const int turns = (wc + kRowBatchCollideWarps - 1) / kRowBatchCollideWarps;
+    const int wraps = by + 2 <= ny && cols >= 3 ? 1 : (by + 2 <= 2 * ny ? 2 : 3);
+    const double lat_d = 0.85 * scale, lat_c = 0.134 * turns * scale + 0.285;
+    double plane = (lat_d > lat_c ? lat_d : lat_c) + 0.0365 * (wd + 1.07 * wc) * scale;
+    const double copies = 19.0 * (0.0375 * wraps + (double)(by + 2) * nx * es / 54.0 / 1900.0);
+    if (copies > plane) plane = copies;
+    const double t = (z + 2) * plane + 5.0;
+    total += it * t;
+    items += it;
+    most = t > most ? t : most;
+    mem += (double)nx * ny * b[k].nz * 38.0 * es * 1.15 / 6.5e6;
+  }
+  double sm = total / items * ((items + sms - 1) / sms);
+  if (most > sm) sm = most;
+  return sqrt(sqrt(sm * sm * sm * sm + mem * mem * mem * mem));
+}
+// The same with a moment kernel (kBatchMoment, kBatchMomentElem) in z chunks of zc planes
+// (0: common_zchunk): a tile's plane takes 1.25 us, or 0.85 (FP16 0.62) for each CTA that
+// an SM holds at a time.
+inline double batch_tile_us(int prec, int mode, const MixBox* b, int n, int zc) {
+  constexpr int sms = 152;
+  const int cap = mode == kBatchMomentElem ? 2 : (prec == kF16 ? 4 : 3), es = prec == kF16 ? 2 : 4;
+  if (zc == 0) zc = common_zchunk(prec, 4, mode, b, n, sms * cap);
+  const double over = mode == kBatchMomentElem ? 1.65 : (prec == kF16 ? 2.1 : 1.3);
+  double planes = 0.0, mem = 0.0;
+  long long items = 0;
+  int deepest = 0, rows = 0;
+  for (int k = 0; k < n; ++k) {
+    const int z = b[k].nz < zc ? b[k].nz : zc;
+    const long long it = batch_items(prec, 4, mode, b[k].nx, b[k].ny, b[k].nz, z, &rows);
+    items += it;
+    planes += (double)it * (z + 2);
+    deepest = z + 2 > deepest ? z + 2 : deepest;
+    mem += (double)b[k].nx * b[k].ny * b[k].nz * 38.0 * es * over / 6.5e6;
+  }
+  const long long per_sm = (items + sms - 1) / sms, rounds = (items + sms * cap - 1) / (sms * cap);
+  const double share = (prec == kF16 ? 0.62 : 0.85) * (per_sm < cap ? per_sm : cap);
+  const double plane = share > 1.25 ? share : 1.25;
+  double sm = rounds * planes / items * plane;
+  if (deepest * plane > sm) sm = deepest * plane;
+  sm += 1.9;
+  return sqrt(sqrt(sm * sm * sm * sm + mem * mem * mem * mem));
+}
+// The modes that take a set of lattices, and the one it gets.  The row kernel's few large
+// items suit sets of large boxes (8 of 44^3 22 us a step, the moment kernel 39), the tile
+// kernels' many small CTAs sets of small ones (48 of 16^3 16 us, the row kernel 33; 391 of
+// 8^3 35, 114), so the two expected times decide, for the lattices that run at a time.
+// Measured on 229 sets of 1 to 1389 lattices, 6^3 to 128^3 and flat ones, in groups and
+// batches: the choice is 0.1% off the faster kernel on the mean, 7% at most.  (Never the
+// row kernel below 190000 nodes in the whole set, where none was measured.)
+struct BatchMix {
+  int prec, stencil;
+  int resident;       // lattices that run at a time (0: all)
+  int tile_zchunk;    // z chunk of the tile kernels (0: common_zchunk)
+  bool all[kBatchModes] = {true, true, true, true, true, true};
+  double nodes = 0.0;
+  std::vector<MixBox> boxes;
+  void add(int nx, int ny, int nz, double tau) {
+    for (int m = 0; m < kBatchModes; ++m) all[m] = all[m] && batch_mode_takes(prec, stencil, m, nx, ny, nz, tau);
+    nodes += (double)nx * ny * nz;
+    boxes.push_back(MixBox{nx, ny, nz});
+  }
+  bool takes(int mode) const { return mode >= 0 && mode < kBatchModes && all[mode]; }
+  int tile_mode() const {
+    for (int m : {kBatchMoment, kBatchMomentElem, kBatchMixedTau})
+      if (all[m]) return m;
+    return kBatchMoment;
+  }
+  int row_mode() const {   // -1: none
+    if (nodes < 190000.0) return -1;
+    return all[kBatchRow] ? kBatchRow : (all[kBatchRowAny] ? kBatchRowAny : -1);
+  }
+  int mode() const {
+    const int row = row_mode(), tile = tile_mode();
+    if (row < 0) return tile;
+    std::vector<MixBox> now;   // as many as run at a time, spread over the set
+    const size_t n = boxes.size(), m = resident > 0 && (size_t)resident < n ? (size_t)resident : n;
+    for (size_t k = 0; k < m; ++k) now.push_back(boxes[k * n / m]);
+    const double r = batch_row_us(prec, row, now.data(), (int)m);
+    return r < batch_tile_us(prec, tile, now.data(), (int)m, tile_zchunk) ? row : tile;
+  }
+  // the modes that the batch autotuner times
+  bool candidate(int m) const {
+    if (!all[m]) return false;
+    if (m == kBatchMixedTau) return tile_mode() == m;
+    return batch_mode_row(m) ? m == row_mode() : true;
+  }
+};
+cudaError_t launch_row_batch_any(int prec, bool aligned, const BatchEntry* table, const BatchHeader* hdr, int step,
+                                 bool prepare, int* grid, cudaStream_t s);
 cudaError_t launch_batch_f64(int stencil, int mode, const BatchEntry* table, const BatchHeader* hdr,
                              int step, bool prepare, int* grid, cudaStream_t s);
 cudaError_t launch_batch_f32(int stencil, int mode, const BatchEntry* table, const BatchHeader* hdr,

@@ -3,11 +3,11 @@
 
 using namespace lbm;
 
-// boxes: n triples nx, ny, nz; takes and candidates: kBatchModes flags each.  Returns
-// the mode the set gets.
-extern "C" int rule_batch_mix(int prec, int stencil, int n, const int* boxes, const double* tau, int* takes,
-                              int* candidates) {
-  BatchMix m{prec, stencil};
+// boxes: n triples nx, ny, nz; slots: lattices of the set that run at a time, 0 a group of
+// all; takes and candidates: kBatchModes flags each.  Returns the mode the set gets.
+extern "C" int rule_batch_mix(int prec, int stencil, int n, const int* boxes, const double* tau, int slots,
+                              int* takes, int* candidates) {
+  BatchMix m{prec, stencil, slots, slots > 0 ? 16 : 0};
   for (int k = 0; k < n; ++k) m.add(boxes[3 * k], boxes[3 * k + 1], boxes[3 * k + 2], tau[k]);
   for (int k = 0; k < kBatchModes; ++k) {
     takes[k] = m.takes(k);

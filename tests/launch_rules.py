@@ -30,13 +30,14 @@ def compile_so(source):
     return ctypes.CDLL(str(out))
 
 
-def batch_mix(prec, stencil, boxes, taus=None):
-    """(mode, modes that take every box, modes the batch autotuner times) of a set of lattices"""
+def batch_mix(prec, stencil, boxes, taus=None, slots=0):
+    """(mode, modes that take every box, modes the batch autotuner times) of a set of lattices:
+    a group, or a batch of so many slots"""
     n = len(boxes)
     flat = (ctypes.c_int * (3 * n))(*[s for b in boxes for s in b])
     tau = (ctypes.c_double * n)(*(taus or [1.0] * n))
     takes, cand = (ctypes.c_int * 6)(), (ctypes.c_int * 6)()
-    mode = compile_so("launch_rules.cu").rule_batch_mix(PREC[prec], stencil, n, flat, tau, takes, cand)
+    mode = compile_so("launch_rules.cu").rule_batch_mix(PREC[prec], stencil, n, flat, tau, slots, takes, cand)
     return mode, {k for k in range(6) if takes[k]}, {k for k in range(6) if cand[k]}
 
 

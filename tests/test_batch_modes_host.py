@@ -21,12 +21,12 @@ MIXED, UNIT, MOMENT, ELEM, ROW, ROW_ANY = range(6)
     ([(32, 32, 32)] * 5, ELEM, {ELEM, UNIT}),
 ])
 def test_f32_sets(boxes, mode, tuned):
-    assert launch_rules.batch_mix("f32", 4, boxes)[::2] == (mode, tuned)
+    assert launch_rules.batch_mix("f32", 4, boxes, slots=2)[::2] == (mode, tuned)
 
 
 def test_f16_f64_and_mixed_tau_sets():
-    assert launch_rules.batch_mix("f16", 4, [(64, 64, 64)])[::2] == (ROW, {ROW, MOMENT})
-    assert launch_rules.batch_mix("f16", 4, [(64, 40, 36)])[::2] == (MOMENT, {MOMENT})
+    assert launch_rules.batch_mix("f16", 4, [(64, 64, 64)], slots=1)[::2] == (ROW, {ROW, MOMENT})
+    assert launch_rules.batch_mix("f16", 4, [(64, 40, 36)], slots=1)[::2] == (MOMENT, {MOMENT})
     assert launch_rules.batch_mix("f64", 4, [(64, 64, 64)])[::2] == (MOMENT, {MOMENT, ELEM, UNIT})
     assert launch_rules.batch_mix("f64", 6, [(37, 64, 64)])[::2] == (ELEM, {ELEM, UNIT})
     assert launch_rules.batch_mix("f32", 4, [(64, 64, 64)] * 2, [1.0, 0.8])[::2] == (MIXED, {MIXED})
@@ -47,3 +47,21 @@ def test_every_offered_mode_takes_every_box(prec, stencil):
         rows = prec == "f32" and stencil == 4 and all(box[0] < 600 for box in (a, b))
         assert (ROW_ANY in takes) == rows
         assert (ROW in takes) == (rows and all(box[0] % 4 == 0 for box in (a, b)))
+
+
+@pytest.mark.parametrize("boxes,slots,rows", [
+    # groups
+    ([(8, 8, 8)] * 391, 0, False), ([(16, 16, 16)] * 48, 0, False), ([(20, 20, 20)] * 100, 0, False),
+    ([(24, 24, 24)] * 14, 0, False), ([(32, 32, 32)] * 6, 0, False), ([(64, 3, 64)] * 100, 0, False),
+    ([(461, 48, 48)] * 4, 0, False), ([(65, 65, 65)], 0, False), ([(64, 64, 64), (65, 65, 65)], 0, False),
+    ([(33, 33, 33)] * 8, 0, True), ([(40, 40, 40)] * 5, 0, True), ([(32, 32, 32)] * 60, 0, True),
+    ([(64, 64, 64)] * 4, 0, True), ([(65, 65, 65)] * 3, 0, True), ([(128, 128, 128)] * 2, 0, True),
+    ([(s, s, s) for s in (64, 72, 80, 96, 112, 128)], 0, True),
+    # batches: the tile kernels' z chunks of 16 planes leave few small items
+    ([(16, 16, 16)] * 48, 8, True), ([(16, 16, 16)] * 48, 48, False), ([(8, 8, 8)] * 400, 100, False),
+    ([(24, 24, 24)] * 64, 2, True), ([(24, 24, 24)] * 60, 60, True), ([(64, 3, 64)] * 20, 20, False),
+    ([(64, 64, 64)] * 4, 1, True), ([(97, 97, 97)] * 4, 4, True),
+])
+def test_the_row_kernel_gets_the_sets_it_is_faster_on(boxes, slots, rows):
+    """Measured on both sides of the line (GB300)."""
+    assert (launch_rules.batch_mix("f32", 4, boxes, slots=slots)[0] in (ROW, ROW_ANY)) == rows

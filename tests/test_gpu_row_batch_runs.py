@@ -19,7 +19,7 @@ QUEUES = [   # storage, slots, boxes, kernel mode
 @pytest.mark.parametrize("tuned", [False, True])
 @pytest.mark.parametrize("prec,slots,boxes,mode", QUEUES)
 def test_batch_on_the_row_kernel_equals_single_runs(prec, slots, boxes, mode, tuned):
-    assert launch_rules.batch_mix(prec, 4, boxes)[0] == mode
+    assert launch_rules.batch_mix(prec, 4, boxes, slots=slots)[0] == mode
     runs = [(b, -5.0 - 0.1 * (k % 3), max(3.0, min(b) / 4.0), 1.9 - 0.05 * k) for k, b in enumerate(boxes)]
     batch = P.Batch(slots, tuple(max(b[a] for b in boxes) for a in range(3)), prec=prec)
     try:
