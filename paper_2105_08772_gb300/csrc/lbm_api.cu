@@ -1450,8 +1450,8 @@ struct lbm_batch {
   int graph_mode = -1;       // BatchMode the graph (and the table's tiling) was made for
   int grid = 0;              // resident CTAs of that mode's kernel
   long long lattice_updates = 0;
-  // configuration chosen by lbm_batch_autotune (defaults: the natural kernel mode,
-  // z chunks of min(16, nz), every slot)
+  // configuration chosen by lbm_batch_autotune (defaults: the natural kernel mode, z
+  // chunks (0) of min(16, nz) planes, the row kernel's evened out; every slot)
   int mode_override = -1;
   int zchunk = 0;
   int slot_cap = 0;
@@ -1778,7 +1778,8 @@ lbm_status lbm_batch_autotune(lbm_batch* b, int reps, long long* choice) {
   const int save_cap = b->slot_cap;
   for (int mode = kBatchModes - 1; mode >= 0; --mode) {
     if (!mix.candidate(mode)) continue;
-    for (int zc : {8, 16, 32}) {
+    for (int zc : {0, 8, 16, 32}) {
+      if (zc == 0 && !batch_mode_row(mode)) continue;   // (the tile kernels' default is 16)
       for (int cap : caps) {
         b->mode_override = mode;
         b->zchunk = zc;
@@ -1791,11 +1792,8 @@ lbm_status lbm_batch_autotune(lbm_batch* b, int reps, long long* choice) {
         std::vector<lbm_ctx*> hidden(b->slots, nullptr);
         for (int k = cap; k < b->slots; ++k) std::swap(hidden[k], b->slot_ctx[k]);
         b->graph_mode = mode;   // the table's tiling follows the kernel launched
-        st = batch_upload(b);
-        int grid = 0;
-        cudaError_t ce = cudaSuccess;
-        if (st == LBM_OK)
-          ce = launch_batch(b->prec, b->stencil, mode, b->table_dev, b->hdr_dev, 0, true, &grid, b->stream);
+        cudaError_t ce = launch_batch(b->prec, b->stencil, mode, b->table_dev, b->hdr_dev, 0, true, &b->grid, b->stream);
+        st = ce == cudaSuccess ? batch_upload(b) : LBM_OK;
         for (int r = 0; r < 2 && st == LBM_OK && ce == cudaSuccess; ++r)
           ce = launch_batch(b->prec, b->stencil, mode, b->table_dev, b->hdr_dev, r & 1, false, nullptr, b->stream);
         if (st == LBM_OK && ce == cudaSuccess) ce = cudaEventRecord(e0, b->stream);
@@ -1851,9 +1849,7 @@ lbm_status lbm_batch_autotune(lbm_batch* b, int reps, long long* choice) {
   if (b->graph) cudaGraphExecDestroy(b->graph);
   b->graph = nullptr;
   b->graph_mode = -1;
-  // (the row kernel reports as the moment kernel that it stands in for)
-  const int shown = best_mode == kBatchRow ? kBatchMoment : (best_mode == kBatchRowAny ? kBatchMomentElem : best_mode);
-  if (choice) *choice = (long long)shown * 1000000 + (long long)best_zc * 1000 + best_cap;
+  if (choice) *choice = (long long)best_mode * 1000000 + (long long)best_zc * 1000 + best_cap;
   return LBM_OK;
 }
 

@@ -24,8 +24,11 @@ def test_batch_on_the_row_kernel_equals_single_runs(prec, slots, boxes, mode, tu
     batch = P.Batch(slots, tuple(max(b[a] for b in boxes) for a in range(3)), prec=prec)
     try:
         ids = [batch.enqueue(b, G=G, R=R, rho_in=ri, rho_out=0.13) for b, G, R, ri in runs]
-        if tuned:
-            batch.autotune(reps=2)
+        if tuned:   # the code names the kernel, of those that take every box
+            code = batch.autotune(reps=2)
+            offered = launch_rules.batch_mix(prec, 4, boxes, slots=slots)[2]
+            assert mode in offered and code // 10 ** 6 in offered
+            assert code // 1000 % 1000 in ((0, 8, 16, 32) if code // 10 ** 6 >= ROW else (8, 16, 32))
         batch.run(max_steps=96, check_every=48, tol_dP_rel=-1.0, tol_du=-1.0)
         for rid, (b, G, R, ri) in zip(ids, runs):
             status, got = batch.result(rid)
