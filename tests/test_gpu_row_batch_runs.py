@@ -13,6 +13,10 @@ KEYS = ("n_in", "n_out", "P_in", "P_out", "dP", "mass", "R_e", "C", "D", "max_u"
 ROW, ROW_ANY = 4, 5
 QUEUES = [   # storage, slots, boxes, kernel mode
     ("f32", 6, [(32, 32, 32)] * 4 + [(16, 64, 64)] * 3, ROW),
+    ("f32", 3, [(64, 64, 64), (48, 40, 36), (72, 56, 31), (96, 24, 50), (40, 64, 64)], ROW),
+    ("f32", 2, [(61, 60, 43), (33, 47, 29), (64, 64, 40), (85, 31, 50)], ROW_ANY),
+    ("f16", 2, [(64, 64, 64), (48, 40, 36), (56, 66, 30), (128, 20, 41)], ROW),
+    ("f16", 3, [(64, 16, 48)] * 4 + [(256, 9, 11)], ROW),
 ]
 
 
