@@ -58,9 +58,9 @@ constexpr int kRowDead = 248;   // byte of the give-up flag (behind the mbarrier
 __host__ __device__ constexpr int row_group_first(int g) { return g == 0 ? 0 : (g == 1 ? 7 : (g == 2 ? 11 : (g == 3 ? 15 : Q))); }
 
 // Shared memory of one row CTA (row_caps gives SLOT, MCAP and KD per storage).
-template <int P_, int ST_>
+template <int P_>
 struct RowShape {
-  static constexpr int P = P_, ST = ST_;
+  static constexpr int P = P_, ST = 4;
   using T = typename Storage<P>::T;
   using S = typename Storage<P>::S;
   static constexpr int R = stencil_radius<ST>();
@@ -72,7 +72,7 @@ struct RowShape {
   static constexpr int VE = 16 / (int)sizeof(S);
   static constexpr int NR = 2 * R + 2;                     // psi planes in the ring
   static constexpr int NM = R + 2;                         // planes of moments
-  static constexpr int PW = sizeof(T) == 4 ? 2 : 1;        // nodes of a packed operand
+  static constexpr int PW = 2;                             // nodes of a packed operand
   static constexpr unsigned head_bytes = 256;              // mbarriers, the give-up flag
   static constexpr unsigned stage_bytes = (unsigned)sizeof(S) * Q * SLOT;
   static constexpr unsigned ring_off = head_bytes + stage_bytes;
@@ -86,12 +86,7 @@ struct RowShape {
   static_assert(smem_bytes <= kMaxSmemPerCta, "one CTA per SM");
 };
 
-template <typename T> struct Pack;
-template <> struct Pack<float> {
-  using V = float2;
-  static __device__ __forceinline__ float get(float2 v, int i) { return i == 0 ? v.x : v.y; }
-  static __device__ __forceinline__ float2 make(float a, float b) { return make_float2(a, b); }
-};
+__device__ __forceinline__ float row_node(float2 v, int w) { return w == 0 ? v.x : v.y; }
 
 __device__ __forceinline__ void row_bulk_copy(void* dst, const void* src, unsigned bytes, unsigned long long* bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
@@ -138,7 +133,7 @@ __device__ __forceinline__ float2 row_ld_pair(const unsigned char* smem, unsigne
   else return row_ld<float2>(smem, off);
 }
 
-// The nodes a thread takes at a time: one packed operand of two (FP64: one).
+// The nodes a thread takes at a time: one packed operand of two.
 // A padded plane's nodes are numbered flat, j = row nx + x, in the population slots,
 // the psi planes and (interior nodes) the moments alike.
 //  * PAIR (aligned rows): two x-neighbours at an even x;
@@ -148,9 +143,8 @@ struct RowNodes {
   static constexpr int P = Sh::P;
   using T = typename Sh::T;
   using S = typename Sh::S;
-  using V = typename Pack<T>::V;
   static constexpr int PW = Sh::PW, R = Sh::R;
-  static constexpr bool PAIR = ALIGNED && PW == 2 && Sh::PAIRS;
+  static constexpr bool PAIR = ALIGNED && Sh::PAIRS;
   static constexpr int NEXT = PAIR ? 1 : 32;    // second node's distance from the first
   static constexpr int NL = PAIR ? 1 : PW;
   int j;               // first node
@@ -158,7 +152,7 @@ struct RowNodes {
 
   // flat index of the first node of a thread's t-th unit, t consecutive over a warp
   static __device__ __forceinline__ int first(int t) {
-    return PW == 1 ? t : (PAIR ? 2 * t : (t & ~31) * 2 + (t & 31));
+    return PAIR ? 2 * t : (t & ~31) * 2 + (t & 31);
   }
   __device__ __forceinline__ void set(int j0, int nx) {
     j = j0;
@@ -176,19 +170,16 @@ struct RowNodes {
   }
 };
 
-// psi of NP packed densities (one branch on its kind for all of them)
-template <typename T, int NP>
-__device__ __forceinline__ void row_psi(typename Pack<T>::V* n, const EosParams& e) {
-  constexpr int PW = sizeof(T) == 4 ? 2 : 1;
-  auto all = [&](auto f) {
-#pragma unroll
-    for (int p = 0; p < NP; ++p)
-      n[p] = Pack<T>::make(f(Pack<T>::get(n[p], 0)), PW == 2 ? f(Pack<T>::get(n[p], 1)) : (T)0);
-  };
+// psi of a packed density, one branch on its kind
+__device__ __forceinline__ float2 row_psi(float2 n, const EosParams& e) {
   EosParams k = e;
-  if (e.kind == kPsiOneMinusExp) { k.kind = kPsiOneMinusExp; all([&](T x) { return psi_of<T>(x, k); }); }
-  else if (e.kind == kPsiExpInv) { k.kind = kPsiExpInv; all([&](T x) { return psi_of<T>(x, k); }); }
-  else { k.kind = kPsiCS; all([&](T x) { return psi_of<T>(x, k); }); }
+  auto both = [&](int kind) {
+    k.kind = kind;
+    return make_float2(psi_of<float>(n.x, k), psi_of<float>(n.y, k));
+  };
+  if (e.kind == kPsiOneMinusExp) return both(kPsiOneMinusExp);
+  if (e.kind == kPsiExpInv) return both(kPsiExpInv);
+  return both(kPsiCS);
 }
 
 // One item: rows [y0, y0 + h), planes [z0, z0 + zc) of lattice d, walked upwards
@@ -200,7 +191,7 @@ __device__ __forceinline__ void row_process_item(const LatticeDesc& d, const Row
   using N = RowNodes<Sh, ALIGNED>;
   using T = typename Sh::T;
   using S = typename Sh::S;
-  using V = typename Pack<T>::V;
+  using V = float2;
   constexpr int P = Sh::P, R = Sh::R, PW = Sh::PW, VE = Sh::VE, SLOT = Sh::SLOT;
   unsigned long long* full = reinterpret_cast<unsigned long long*>(smem);
   unsigned long long* empty = full + kRowGroups;
@@ -337,7 +328,7 @@ __device__ __forceinline__ void row_process_item(const LatticeDesc& d, const Row
         for (int w = 0; w < PW; ++w)
           v[w] = staged_value<P>(row_ld<S>(smem, slot + (unsigned)(nd[k].at(w, -cx(i)) * (int)sizeof(S)) +
                                                      (ALIGNED ? 0u : dy[ALIGNED ? 0 : k][w][cy(i) + 1])));
-        return Pack<T>::make(v[0], v[1]);
+        return make_float2(v[0], v[1]);
       };
       auto wait = [&](int g) { row_wait(full + g, use & 1, dead); };
       auto done = [&](int g) {
@@ -404,11 +395,10 @@ __device__ __forceinline__ void row_process_item(const LatticeDesc& d, const Row
           jy[k] = vmul(jy[k], is);
           jz[k] = vmul(jz[k], is);
         }
-        V n = vadd(Lane<V>::all(n0), dn);
-        row_psi<T, 1>(&n, d.eos);
+        const V psi = row_psi(vadd(Lane<V>::all(n0), dn), d.eos);
         const int f = nd[k].j, m = f - R * nx;     // m: interior index (halo rows keep psi only)
         if constexpr (N::PAIR) {   // a pair is whole: in the plane or not, interior or not
-          if (f < nodes) *reinterpret_cast<V*>(smem + ring + (unsigned)(f * 4)) = n;
+          if (f < nodes) *reinterpret_cast<V*>(smem + ring + (unsigned)(f * 4)) = psi;
           if (m >= 0 && m < h * nx) {
             unsigned char* const to = smem + mq + (unsigned)(m * 4);
             *reinterpret_cast<V*>(to) = dn;
@@ -420,14 +410,14 @@ __device__ __forceinline__ void row_process_item(const LatticeDesc& d, const Row
 #pragma unroll
           for (int w = 0; w < PW; ++w) {
             if (f + w * N::NEXT >= nodes) continue;
-            *reinterpret_cast<T*>(smem + ring + (unsigned)((f + w * N::NEXT) * (int)sizeof(T))) = Pack<T>::get(n, w);
+            *reinterpret_cast<T*>(smem + ring + (unsigned)((f + w * N::NEXT) * (int)sizeof(T))) = row_node(psi, w);
             const int mw = m + w * N::NEXT;
             if (mw < 0 || mw >= h * nx) continue;
             unsigned char* const to = smem + mq + (unsigned)(mw * (int)sizeof(T));
-            *reinterpret_cast<T*>(to) = Pack<T>::get(dn, w);
-            *reinterpret_cast<T*>(to + Sh::comp_bytes) = Pack<T>::get(jx[k], w);
-            *reinterpret_cast<T*>(to + 2 * Sh::comp_bytes) = Pack<T>::get(jy[k], w);
-            *reinterpret_cast<T*>(to + 3 * Sh::comp_bytes) = Pack<T>::get(jz[k], w);
+            *reinterpret_cast<T*>(to) = row_node(dn, w);
+            *reinterpret_cast<T*>(to + Sh::comp_bytes) = row_node(jx[k], w);
+            *reinterpret_cast<T*>(to + 2 * Sh::comp_bytes) = row_node(jy[k], w);
+            *reinterpret_cast<T*>(to + 3 * Sh::comp_bytes) = row_node(jz[k], w);
           }
         }
       }
@@ -492,20 +482,20 @@ __device__ __forceinline__ void row_process_item(const LatticeDesc& d, const Row
         const unsigned row = pl[dz + R][dy + R];
         if constexpr (N::PAIR) {
           if (dx == 0) return row_ld<V>(smem, row + jc);
-          if (dx < 0) return Pack<T>::make(row_ld<T>(smem, row + xl[0]), row_ld<T>(smem, row + jc));
-          return Pack<T>::make(row_ld<T>(smem, row + jc + (unsigned)sizeof(T)), row_ld<T>(smem, row + xr[PW - 1]));
+          if (dx < 0) return make_float2(row_ld<T>(smem, row + xl[0]), row_ld<T>(smem, row + jc));
+          return make_float2(row_ld<T>(smem, row + jc + (unsigned)sizeof(T)), row_ld<T>(smem, row + xr[PW - 1]));
         } else {
           T v[2] = {(T)0, (T)0};
 #pragma unroll
           for (int w = 0; w < PW; ++w)
             v[w] = row_ld<T>(smem, row + (dx == 0 ? jc + (unsigned)(w * N::NEXT * (int)sizeof(T)) : dx > 0 ? xr[w] : xl[w]));
-          return Pack<T>::make(v[0], v[1]);
+          return make_float2(v[0], v[1]);
         }
       };
       auto moment = [&](int comp) {
         const unsigned off = mq + comp * Sh::comp_bytes + (unsigned)(f * (int)sizeof(T));
         if constexpr (N::PAIR) return row_ld<V>(smem, off);
-        else return Pack<T>::make(row_ld<T>(smem, off), PW == 2 ? row_ld<T>(smem, off + N::NEXT * (unsigned)sizeof(T)) : (T)0);
+        else return make_float2(row_ld<T>(smem, off), row_ld<T>(smem, off + N::NEXT * (unsigned)sizeof(T)));
       };
       V Fx, Fy, Fz;
       sc_force_at<V, Sh::ST>(at, at(0, 0, 0), G, Fx, Fy, Fz);
@@ -527,8 +517,8 @@ __device__ __forceinline__ void row_process_item(const LatticeDesc& d, const Row
                 if constexpr (P == kF16) *reinterpret_cast<__half*>(at) = __float2half_rn(v);
                 else *reinterpret_cast<T*>(at) = v;
               };
-              put(to, Pack<T>::get(g, 0));
-              if (PW == 2 && ok1) put(to + N::NEXT * sizeof(S), Pack<T>::get(g, 1));
+              put(to, row_node(g, 0));
+              if (ok1) put(to + N::NEXT * sizeof(S), row_node(g, 1));
             }
           });
     }

@@ -9,7 +9,7 @@ namespace lbm {
 // 128^3 58.5 -> 56.2 us, 64^3 17.8 -> 15.2 us when it came in).
 template <int P, bool ALIGNED>
 static cudaError_t launch_row_shape(const LatticeDesc& d, const RowPlan* r, cudaStream_t s) {
-  using Sh = RowShape<P, 4>;
+  using Sh = RowShape<P>;
   auto kern = lattice_row_kernel<Sh, ALIGNED>;
   if (!r)   // prepare
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::smem_bytes);
@@ -39,7 +39,7 @@ static cudaError_t launch_row(const LatticeDesc& d, bool prepare, cudaStream_t s
 template <int P, bool ALIGNED>
 static cudaError_t launch_row_batch(const BatchEntry* table, const BatchHeader* hdr, int step, bool prepare,
                                     int* grid, cudaStream_t s) {
-  using Sh = RowShape<P, 4>;
+  using Sh = RowShape<P>;
   auto kern = lattice_row_batch_kernel<Sh, ALIGNED>;
   static int sms = 0;
   if (prepare || sms == 0) {
