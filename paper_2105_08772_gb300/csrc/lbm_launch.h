@@ -129,9 +129,12 @@ constexpr size_t kMaxSmemPerCta = 227 * 1024;   // opt-in limit of one CTA on sm
 
 // ---------------------------------------------------------------- row kernel
 // The whole-row step (lbm_kernels_row.cuh) behind tile kinds 5 and 6 with a
-// launcher-chosen z chunk at tau = 1.  One CTA of at most kRowThreads threads (128
-// registers each: the kernel must not spill, a few spilled words in its plane loop
-// cost it a third) and nearly all of an SM's shared memory per SM.
+// launcher-chosen z chunk at tau = 1.  One CTA of at most kRowThreads threads and
+// nearly all of an SM's shared memory per SM: 128 registers a thread.  Versions whose
+// plane loop spilled 16 bytes and more were 10 to 40% slower (L1 is some 20 KB beside
+// that much shared memory).  The FP16 kernels and the FP32 one for aligned rows spill
+// nothing; a few words still spill in the FP32 ones for any rows (12 bytes) and for
+// batches (aligned rows 24 bytes, any rows 52).
 constexpr int kRowThreads = 512;
 
 // How one launch cuts a lattice.

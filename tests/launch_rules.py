@@ -13,12 +13,18 @@ ROOT = Path(__file__).resolve().parents[1]
 PREC = {"f64": 0, "f32": 1, "f16": 2}
 
 
-@functools.lru_cache(maxsize=None)
-def compile_so(source):
-    """tests/<source> compiled with the library's flags and loaded"""
+def build_module():
+    """the package's build.py, loaded by path"""
     spec = importlib.util.spec_from_file_location("_lbm_build_for_rules", ROOT / "paper_2105_08772_gb300" / "build.py")
     b = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(b)
+    return b
+
+
+@functools.lru_cache(maxsize=None)
+def compile_so(source):
+    """tests/<source> compiled with the library's flags and loaded"""
+    b = build_module()
     try:
         nvcc = b.nvcc()
     except RuntimeError:
