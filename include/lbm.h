@@ -238,10 +238,12 @@ lbm_status lbm_autotune(lbm_ctx* ctx, int reps, long long* choice);
  * for 32 x 8 tiles with E4 (depth 1, and depth 2 in F32) and 32 x 4 with E6/E8
  * (depth 1).  Kind 5 also takes F16 storage (E4, 32 x 8 tiles, tau = 1,
  * nx % 8 == 0, nx >= 48).  Kinds 5 and 6 with z chunk 0 stand for the fastest
- * kernel of the box: the whole-row kernel (E4, tau = 1, F32 and F16, from some
- * 200000 to 1200000 nodes on, rows of up to 597 / 768 nodes), the step in two passes
- * (F64; F32 with E6 / E8, tau != 1 or smaller boxes), else the kernel of that name; with a z chunk
- * given, always the kernel of that name.  The default (lbm_create) is kind 5 where it
+ * kernel of the box: the whole-row kernel (E4, tau = 1; F32 from 350000 nodes on,
+ * 1200000 where nx % 4 != 0, F16 from 190000; rows of up to 597 / 768 nodes; where it
+ * is expected to be the faster one), the step in two passes (F64; F32 with E6, with E8 at
+ * tau = 1, else up to 1500000 nodes, in calls of lbm_step with fewer than 128 steps not
+ * for the smallest boxes), else the kernel of that name; with a z chunk given, always the
+ * kernel of that name.  The default (lbm_create) is kind 5 where it
  * applies, else kind 6, else kind 1 (kind 5 or 0 for F16).  A code that is not compiled
  * for this context's precision, stencil and box gives LBM_EINVAL.  lbm_get_tile
  * returns the current code.  In F32/F64 storage results do not depend on the

@@ -1,8 +1,9 @@
 // Unit-relaxation-time variant of the pipelined Shan-Chen step.  Without a fixed z
-// chunk FP32 and FP64 boxes take the row kernel (lbm_kernels_row.cuh) or the two passes
-// (lbm_kernels_split.cuh) but for large FP32 boxes whose rows are too long for an item,
-// FP16 boxes below 190000 nodes are this kernel's; it also runs the batches that the
-// row batch kernel does not take.
+// chunk FP64 boxes take the two passes (lbm_kernels_split.cuh), FP32 and FP16 boxes the
+// row kernel (lbm_kernels_row.cuh) where it is the faster one (row_pays) and FP32 boxes up
+// to 1.5 million nodes else the two passes.  This kernel's are the rest: large FP32 boxes
+// whose rows are too long for an item or whose x-y planes are small, small FP16 boxes, and
+// the batches and groups of small lattices (BatchMix).
 //
 // With tau = 1 the BGK update of Eq. (4) loses its f_i term:
 //     f*_i = f_i - (f_i - f_i^eq) + F_i = f_i^eq(n, u) + F_i,
