@@ -409,7 +409,7 @@ lbm_status plan_rows(lbm_ctx* c) {
     int dev = 0, sms = 0;
     LBM_CUDA(c, cudaGetDevice(&dev));
     LBM_CUDA(c, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    c->rows = row_plan(c->prec, c->box.nx, c->box.ny, c->box.nz, sms);
+    c->rows = row_plan(c->prec, c->box.nx, c->box.ny, c->box.nz, sms, c->aux != nullptr);
   }
   c->rows_planned = true;
   return LBM_OK;

@@ -174,15 +174,18 @@ struct RowPlan {
 // each and their bytes at 54 per clock, several times as many where the blocks wrap
 // around a short box in y (64x3x5000 67 us, the moment kernel 38).  One-row FP16 items
 // (rows past 576 nodes, densities formed three times) count for a third more.  The
-// others: the two passes (FP32 up to 1.5 million nodes) 28 nodes a nanosecond (30 in a
+// others: the two passes (FP32 up to 1.5 million nodes, where the lattice has the psi
+// plane for them: `passes`) 28 nodes a nanosecond (30 in a
 // replayed graph, but two launches where steps are launched one by one: 64x64x100 13.2 us
 // in rows, 13.5, and 13.7 against 18.6 launched singly); the moment kernel 27 (aligned
-// rows), 23 (any rows; odd boxes), in FP32 its last tile of a row counted whole.
+// rows), 23 (any rows; odd boxes), 22 in boxes that would take the two passes if they
+// could (72^3 21.5 us, 452x30x30 21.2), in FP32 its last tile of a row counted whole.
 // Measured on 456 boxes of 3 to 1389 rows and 3 to 31250 planes: the choice is 0.4% off
 // the faster kernel on the mean, 13% at most; with the row kernel wherever it has a cut it
 // was 9% on the mean and up to 3.5 times (us, row kernel / other: 33x3x20000 502 / 144,
 // 449x80x80 142 / 108, 96x16x4461 240 / 194, F16 600x64x64 64.7 / 54.8).
-inline bool row_pays(int prec, int nx, int ny, int nz, int sms, const RowPlan& r, double plane, double mem) {
+inline bool row_pays(int prec, int nx, int ny, int nz, int sms, bool passes, const RowPlan& r, double plane,
+                     double mem) {
   constexpr int R = 1;
   const double nodes = (double)nx * ny * nz;
   const int by = r.cfg.by, zc = r.cfg.zc, es = prec == kF16 ? 2 : 4;
@@ -196,8 +199,9 @@ inline bool row_pays(int prec, int nx, int ny, int nz, int sms, const RowPlan& r
     if (by == 1) t *= 1.35;
     return t < nodes / 27e3;
   }
-  if (nodes <= 1.5e6) return t < nodes / 28e3;
-  return t < (double)((nx + 31) / 32 * 32) * ny * nz / (r.aligned ? 27e3 : 23e3);
+  if (passes && nodes <= 1.5e6) return t < nodes / 28e3;
+  const double rate = nodes <= 1.5e6 ? 22e3 : (r.aligned ? 27e3 : 23e3);
+  return t < (double)((nx + 31) / 32 * 32) * ny * nz / rate;
 }
 
 // The cut with the least expected time, or ok = false where no item fits (rows too
@@ -213,7 +217,7 @@ inline bool row_pays(int prec, int nx, int ny, int nz, int sms, const RowPlan& r
 // them: the plan's choice is within 4% of the best cut of each, but for two FP16 boxes
 // (128^3 9%, 160^3 10%).  There is no plan where the other kernel is expected to be
 // faster (row_pays).
-inline RowPlan row_plan(int prec, int nx, int ny, int nz, int sms) {
+inline RowPlan row_plan(int prec, int nx, int ny, int nz, int sms, bool passes) {
   constexpr int R = 1;   // E4 (E6 in rows: 256^3 730 us, the two passes 545)
   RowPlan best{false, false, 0, 0, {0, 0, 0, 0}};
   const int es = prec == kF16 ? 2 : 4, ve = 16 / es;
@@ -254,7 +258,7 @@ inline RowPlan row_plan(int prec, int nx, int ny, int nz, int sms) {
       if (zc == 1) break;
     }
   }
-  if (best.ok && !row_pays(prec, nx, ny, nz, sms, best, best_plane, best_mem)) best.ok = false;
+  if (best.ok && !row_pays(prec, nx, ny, nz, sms, passes, best, best_plane, best_mem)) best.ok = false;
   return best;
 }
 

@@ -16,9 +16,10 @@ extern "C" int rule_batch_mix(int prec, int stencil, int n, const int* boxes, co
   return m.mode();
 }
 
-// out: ok, aligned, items, grid, by, zc, density threads, collision threads
-extern "C" void rule_row_plan(int prec, int nx, int ny, int nz, int sms, int* out) {
-  const RowPlan r = row_plan(prec, nx, ny, nz, sms);
+// passes: the lattice has the psi plane of the two passes; out: ok, aligned, items, grid,
+// by, zc, density threads, collision threads
+extern "C" void rule_row_plan(int prec, int nx, int ny, int nz, int sms, int passes, int* out) {
+  const RowPlan r = row_plan(prec, nx, ny, nz, sms, passes != 0);
   const int v[8] = {r.ok, r.aligned, r.items, r.grid, r.cfg.by, r.cfg.zc, r.cfg.nd, r.cfg.nc};
   for (int k = 0; k < 8; ++k) out[k] = v[k];
 }
@@ -34,7 +35,7 @@ extern "C" void rule_row_caps(int prec, int* out) {
 
 // the route of a default step (kind 5 or 6, launcher-chosen z chunk), with a psi plane
 extern "C" int rule_step_route(int prec, int stencil, int unit_tau, int nx, int ny, int nz, int eager) {
-  const RowPlan r = row_plan(prec, nx, ny, nz, 152);
+  const RowPlan r = row_plan(prec, nx, ny, nz, 152, prec != kF16);
   LatticeDesc d{};
   d.nx = nx;
   d.ny = ny;

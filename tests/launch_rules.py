@@ -47,10 +47,10 @@ def batch_mix(prec, stencil, boxes, taus=None, slots=0):
     return mode, {k for k in range(6) if takes[k]}, {k for k in range(6) if cand[k]}
 
 
-def row_plan(prec, box, sms=152):
-    """the row kernel's cut of a box as a dict, or None"""
+def row_plan(prec, box, sms=152, passes=True):
+    """the row kernel's cut of a box as a dict, or None; passes: the lattice has a psi plane"""
     out = (ctypes.c_int * 8)()
-    compile_so("launch_rules.cu").rule_row_plan(PREC[prec], *box, sms, out)
+    compile_so("launch_rules.cu").rule_row_plan(PREC[prec], *box, sms, int(passes), out)
     keys = ("ok", "aligned", "items", "grid", "by", "zc", "nd", "nc")
     return dict(zip(keys, out)) if out[0] else None
 

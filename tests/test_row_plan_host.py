@@ -103,3 +103,11 @@ def test_where_the_row_kernel_pays(prec, box, planned):
     """Measured on both sides of the line (GB300): the row kernel has a plan only where it is
     the faster one."""
     assert (launch_rules.row_plan(prec, box) is not None) == planned
+
+
+@pytest.mark.parametrize("box", [(76, 72, 70), (440, 30, 28), (512, 40, 40)])
+def test_without_the_psi_plane_rows_are_held_against_the_tile_kernels(box):
+    """Boxes that the two passes take from the row kernel, where the workspace has no room
+    for them: the moment kernel is slower than rows there."""
+    assert launch_rules.row_plan("f32", box) is None
+    assert launch_rules.row_plan("f32", box, passes=False)
